@@ -876,7 +876,7 @@ int fdlb_forward_ckpt(fdlb_ctx* c, int64_t nsteps, int every, void* ckpt) {
       e = cudaMemcpyAsync(ck + (s / every) * bytes, c->dp.F, bytes, cudaMemcpyDeviceToDevice, c->stream);
     if (s == nsteps || e != cudaSuccess) break;
     for (int st : {fdlb::kStage3, fdlb::kStage4, fdlb::kFinal}) {
-      int le = fdlb::ctx_launch_stage(c, st, c->stream);
+      int le = fdlb::launch_stage(c->dp, st, c->stream);
       if (le) {
         e = (cudaError_t)le;
         break;

@@ -181,6 +181,7 @@ bool stage_coefficients(const fdlb_tableau& t, double lam, fdlb::StageCoef* sc, 
   const double d1 = e[0];
   const double d2 = e[1] * (1.0 - A(1, 0) * d1);
   sc->c2 = 1.0 - A(1, 0) * d1 - A(1, 1) * d2;
+  sc->c2m1 = A(1, 0) * d1 + A(1, 1) * d2;
   sc->k3 = A(2, 0) * d1 + A(2, 1) * d2;
   sc->k4 = A(3, 0) * d1 + A(3, 1) * d2;
   sc->kf = t.w[0] * d1 + t.w[1] * d2;
@@ -397,6 +398,7 @@ int params_for(const fdlb_grid* grid, int Qphi, int Qchi, double gamma, double t
   double wp[kMaxQ], wc[kMaxQ];
   if (!gauss_hermite(Qphi, p.pp, wp) || !gauss_hermite(Qchi, p.pc, wc))
     return set_err(nullptr, FDLB_EINVAL, "Gauss-Hermite rule failed to converge");
+  for (int k = 0; k < Qphi; ++k) p.pp2[k] = p.pp[k] * p.pp[k];
   weighted_hermite_table(Qphi, p.pp, wp, p.wHp);
   weighted_hermite_table(Qchi, p.pc, wc, p.wHc);
   for (int i = 0; i < kMaxQ * kMaxQ; ++i) {
@@ -436,10 +438,9 @@ int params_for(const fdlb_grid* grid, int Qphi, int Qchi, double gamma, double t
 // Record a context-less error for fdlb_last_error(NULL).
 int record_error(int code, const char* msg) { return set_err(nullptr, code, "%s", msg); }
 
-// Error recording, preparation and stage launch for the other host files.
+// Error recording and preparation for the other host files.
 int ctx_error(fdlb_ctx* c, int code, const char* msg) { return set_err(c, code, "%s", msg); }
 int ctx_prepare(fdlb_ctx* c) { return ensure_prepared(c); }
-int ctx_launch_stage(fdlb_ctx* c, int stage, cudaStream_t s) { return launch_stage_any(c, stage, s); }
 
 }  // namespace fdlb
 
@@ -524,6 +525,7 @@ int fdlb_create(const fdlb_grid* grid, int Qphi, int Qchi, double gamma, double 
     delete c;
     return set_err(nullptr, FDLB_EINVAL, "Gauss-Hermite rule failed to converge");
   }
+  for (int k = 0; k < Qphi; ++k) p.pp2[k] = p.pp[k] * p.pp[k];
   weighted_hermite_table(Qphi, p.pp, wp, p.wHp);
   weighted_hermite_table(Qchi, p.pc, wc, p.wHc);
   for (int i = 0; i < kMaxQ * kMaxQ; ++i) {

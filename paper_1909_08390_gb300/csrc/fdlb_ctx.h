@@ -47,6 +47,5 @@ struct fdlb_ctx {
 namespace fdlb {
 int ctx_error(fdlb_ctx* c, int code, const char* msg);
 int ctx_prepare(fdlb_ctx* c);
-int ctx_launch_stage(fdlb_ctx* c, int stage, cudaStream_t s);
 }  // namespace fdlb
 

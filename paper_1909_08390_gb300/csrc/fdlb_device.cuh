@@ -71,18 +71,6 @@ inline int tile_cells_1d(int variant) {
   }
 }
 
-// Shared memory of one tile: the advected populations of a group on tile +
-// halo, and the interface values along x and y.
-template <int DIM, typename S, int VAR>
-struct TileSmem {
-  using C = TileCfg<DIM, VAR>;
-  static constexpr int SX = C::TX + 2 * 5 + (DIM == 2 ? 1 : 0);  // padded row pitch (2-D)
-  static constexpr int SY = DIM == 2 ? C::TY + 2 * 5 : 1;
-  S tile[C::G][SY][SX];
-  S hx[C::G][C::TY][C::TX + 1];
-  S hy[DIM == 2 ? C::G : 1][DIM == 2 ? C::TX : 1][C::TY + 1];
-};
-
 // Where a tile lives: its problem's size, first cell in the population
 // arrays, and gas and grid constants.
 struct Geo {

@@ -27,6 +27,7 @@ struct StageCoef {
   double a33e3, a43e3, w3e3;    // weights of D3
   double a44e4, w4e4;           // weights of D4
   double c2;                    // F2 = F_eq + c2 (F - F_eq)
+  double c2m1;                  // 1 - c2: F2 = F - (1 - c2) (F - F_eq)
 };
 
 // One 1-D problem of a batch (fdlb_create_batch): its cells occupy
@@ -70,6 +71,7 @@ struct DevParams {
   double DK, kchi;              // D + K and D + K - d
   double dtdx, dtdy;            // dt/dx, dt/dy
   double pp[kMaxQ], pc[kMaxQ];  // phi and chi momenta (ascending)
+  double pp2[kMaxQ];            // squares of the phi momenta
   double wHp[kMaxQ * kMaxQ];    // [l*kMaxQ + k] = w_k He_l(p_k)/l!, phi axis
   double wHc[kMaxQ * kMaxQ];    // same for the chi axis
   // the same tables as binary32 pairs hi + lo (the mixed path's records)

@@ -6,11 +6,11 @@
 //   pass 1  for each group of G populations: stage the advected array on the
 //           tile plus its 5-cell MP-9 halo in shared memory (ghosts by index
 //           clamp = outlet copies of the adjacent fluid node, Sec. IV), march
-//           every tile line computing each interface value once (MP-9 + MP
-//           limiter, fdlb_mp9.cuh), form the flux difference and the explicit
-//           part R_i of the stage (Eq. IMEX), accumulate the moments of R_i
-//           per cell (Eq. Moments_discrete) and park R_i and the running
-//           accumulators in the output arrays;
+//           every tile line (MP-9 + MP limiter; 2-D in 64-bit fixed point,
+//           fdlb_mp9i.cuh, 1-D in binary64, fdlb_mp9.cuh), form the flux
+//           difference and the explicit part R_i of the stage (Eq. IMEX),
+//           accumulate the moments of R_i per cell (Eq. Moments_discrete) and
+//           park R_i and the running accumulators in the output arrays;
 //   pass 2  per cell: n, u, T from the moments, the Hermite equilibrium
 //           factors (Eq. gExpanded, recurrence form), and the closed-form
 //           implicit BGK relaxation of every population (Sec. III).  Stages
@@ -19,227 +19,570 @@
 //           rewrites the relaxed populations and D only.
 // The flux itself never goes to global memory.
 #include "fdlb_device.cuh"
+#include "fdlb_mp9i.cuh"
 
 namespace fdlb {
 namespace {
 
-// One tile (origin x0, y0 of problem g) of one fused stage; see the file
-// header for the two passes.  Ends with every thread past its last use of
-// the shared memory, so a persistent CTA may start its next tile at once.
-template <int DIM, int QP, int QC, int STAGE, typename S, int VAR>
-__device__ __forceinline__ void stage_tile(const DevParams& p, const Geo& geo, int x0, int y0,
-                                           TileSmem<DIM, S, VAR>& sm) {
-  using C = TileCfg<DIM, VAR>;
-  using L = Lat<DIM, QP, QC>;
-  constexpr int TX = C::TX, TY = C::TY, NT = C::NT, G = C::G, SEG = C::SEG;
-  constexpr int SX = TileSmem<DIM, S, VAR>::SX;
-  constexpr int CELLS = TX * TY;
-  constexpr int CPT = (CELLS + NT - 1) / NT;
-  constexpr int NSEG = (TX + 1) / SEG;  // segments per line
-  static_assert(NSEG * SEG == TX + 1, "segments tile the line");
-  constexpr int NLINE = DIM == 2 ? TX + TY : 1;
-  static_assert(G * NLINE * NSEG == NT, "one march task per thread");
+// ---- pass 2 of a cell --------------------------------------------------------
 
-  constexpr int SY = TileSmem<DIM, S, VAR>::SY;
-  auto& tile = sm.tile;
-  auto& hx = sm.hx;
-  auto& hy = sm.hy;
-  S* __restrict__ const F = (S*)p.F;
-  S* __restrict__ const F2 = (S*)p.F2;
-  S* __restrict__ const F3 = (S*)p.F3;
-  S* __restrict__ const A4 = (S*)p.A4;
-  S* __restrict__ const Af = (S*)p.Af;
-  S* __restrict__ const Dn = (S*)p.D;
-
-  const int tid = threadIdx.x;
-  const int64_t N = p.N;  // population stride
-
-  int lxs[CPT], lys[CPT];
-  int64_t cell[CPT];
-  bool valid[CPT];
+// n, u, T of the moment sums, the equilibrium's factors, and row by row of
+// their outer product (1-D: phi, then chi) D = R - F_eq(R) and the relaxed
+// value R - kd D, the next row's values loaded before this row is computed:
+//   stage 3   R3 -> F3 and D3 (in D, free until the final stage rewrites it;
+//             stage 4 applies its terms to A4 and A_fin),
+//   stage 4   R4 -> F4 (in A4) and D4 for the final stage,
+//   final and preparation   F -> F2 and D of the new state.
+// fac (2-D): QP + QC shared doubles of stride FS for this thread's y factors,
+// picked by row at run time (one copy of the row body: code size).
+template <int DIM, int QP, int QC, int STAGE, int FS>
+__device__ __forceinline__ void relax_cell64(const DevParams& p, const Geo& geo, unsigned c,
+                                             const Moments& m, double* fac) {
+  const int64_t N = p.N;
+  const double* __restrict__ const Rin =
+      (const double*)(STAGE == kStage3 ? p.F3 : STAGE == kStage4 ? p.A4 : p.F);
+  double* __restrict__ const Fout =
+      (double*)(STAGE == kStage3 ? p.F3 : STAGE == kStage4 ? p.A4 : p.F2);
+  double* __restrict__ const Dn = (double*)p.D;
+  const StageCoef& sc = p.sc;
+  const double kd = STAGE == kStage3 ? sc.a33e3 : STAGE == kStage4 ? sc.a44e4 : sc.c2m1;
+  constexpr int W = QP > QC ? QP : QC;
+  double cur[W], nxt[W];
 #pragma unroll
-  for (int k = 0; k < CPT; ++k) {
-    const int c = tid + k * NT;
-    lxs[k] = c % TX;
-    lys[k] = c / TX;
-    const int x = x0 + lxs[k], y = y0 + lys[k];
-    valid[k] = (c < CELLS) && (x < geo.nx) && (y < geo.ny);
-    cell[k] = geo.base + (int64_t)y * geo.nx + x;
+  for (int j = 0; j < QP; ++j) cur[j] = (Rin + j * N)[c];
+  double n, ux, uy, T;
+  if (!moments_to_nut<DIM>(geo.invDK, m, n, ux, uy, T)) {
+    atomicOr(p.status, 1u);
+    if (geo.prob >= 0) atomicOr(&p.pstatus[geo.prob], 1u);
   }
-  typename MomAcc<S>::type mom[CPT];
+  // populations p0 .. of a row: D = R - F_eq, F_eq = h f, one fused operation
+  // except in 1-D where F2 needs F_eq itself (small_stage_kernel does the same)
+  auto relax_row = [&](int p0, int nq, const double* h, double f) {
 #pragma unroll
-  for (int k = 0; k < CPT; ++k) mom[k] = {};
-
-  const CoefS<S> sc(p.sc);
-
-  if (STAGE == kPrep) {
-    for (int pop = 0; pop < L::P; ++pop) {
-#pragma unroll
-      for (int k = 0; k < CPT; ++k)
-        if (valid[k]) accumulate<DIM, QP, QC>(p, mom[k], pop, F[pop * N + cell[k]]);
-    }
-  } else {
-    const S* __restrict__ adv = (STAGE == kStage3) ? F2 : (STAGE == kStage4) ? F3 : A4;
-    // this thread's march task: population tg of the group, line, segment
-    const int tg = tid / (NLINE * NSEG);
-    const int tline = (tid / NSEG) % NLINE;
-    // this thread's staged cells (tile offset, cell offset from geo.base or
-    // -1): ghosts by index clamp or wrap; the 2-D halo corners feed no line
-    constexpr int SXH = TX + 2 * H;
-    constexpr int NST = SY * SXH;
-    constexpr int J = (NST + NT - 1) / NT;
-    int soff[J], goff[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const int e = tid + j * NT;
-      const int r = e / SXH, c = e % SXH;
-      soff[j] = r * SX + c;
-      goff[j] = -1;
-      const bool corner = DIM == 2 && (r < H || r >= H + TY) && (c < H || c >= H + TX);
-      if (e < NST && !corner) {
-        const int gx = wrap_or_clamp(x0 - H + c, geo.nx, p.bc);
-        const int gy = (DIM == 2) ? wrap_or_clamp(y0 - H + r, geo.ny, p.bc) : 0;
-        goff[j] = gy * geo.nx + gx;
-      }
-    }
-    // the group's advected populations on tile + halo, copied asynchronously;
-    // the next group's copies run during this group's pass 1
-    auto prefetch = [&](int gfirst) {
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const int pop = gfirst + g;
-        if (pop >= L::P) break;
-        const S* __restrict__ src = adv + (int64_t)pop * N + geo.base;
-#pragma unroll
-        for (int j = 0; j < J; ++j)
-          if (goff[j] >= 0) cp_async(&tile[g][0][0] + soff[j], src + goff[j]);
-      }
-      cp_async_commit();
-    };
-    prefetch(0);
-    for (int g0 = 0; g0 < L::P; g0 += G) {
-      cp_async_wait_all();
-      __syncthreads();  // the group's tile is in; the previous pass 1 is done
-      // ---- every interface value once, marching upwind -> downwind
-      {
-        const int pop = g0 + tg;
-        const bool xline = (DIM == 1) || (tline < TY);
-        const double pv = (pop < L::P) ? (xline ? p.px[pop] : p.py[pop]) : 0.0;
-        const int sgn = (pv >= 0.0) ? 1 : -1;
-        // one call site for x and y lines (a warp holds both kinds): the line
-        // is (base, signed element stride) in the tile and its output slots
-        // (march_task: interface i lies between tile cells i-1 and i, tile
-        // cell c at column/row c + H, mirror image for p < 0)
-        const MarchTask t = march_task(tid, DIM, TX, TY, SEG, SX, sgn);
-        S* out = t.xline ? &hx[tg][t.orow][t.ofirst] : &hy[tg][t.orow][t.ofirst];
-        mp9_march<SEG>(&tile[tg][t.br][t.bc_], t.stride, out, sgn);
-      }
-      __syncthreads();  // the march is done with the tile
-      if (g0 + G < L::P) prefetch(g0 + G);
-      // ---- flux difference, explicit part, moments (pass 1)
-#pragma unroll
-      for (int k = 0; k < CPT; ++k) {
-        if (!valid[k]) continue;
-        const int lx = lxs[k], ly = lys[k];
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-          const int pop = g0 + g;
-          if (pop >= L::P) break;
-          // X = dt * (p . grad F) = dt p_x (Fhat_{x+1/2} - Fhat_{x-1/2})/dx + (y);
-          // single problems use the host's dt p/dx (the same product)
-          const double cxv = geo.prob < 0 ? p.cx[pop] : geo.dtdx * p.px[pop];
-          S X = (S)cxv * (hx[g][ly][lx + 1] - hx[g][ly][lx]);
-          if constexpr (DIM == 2) {
-            const double cyv = geo.prob < 0 ? p.cy[pop] : geo.dtdy * p.py[pop];
-            X = sfma((S)cyv, hy[g][lx][ly + 1] - hy[g][lx][ly], X);
-          }
-          const int64_t e = pop * N + cell[k];
-          S R;
-          if (STAGE == kStage3) {
-            const S f = F[e], dd = Dn[e];
-            R = sfma(-sc.at32, X, sfma(-sc.k3, dd, f));
-            F3[e] = R;
-            A4[e] = sfma(-sc.at42, X, sfma(-sc.k4, dd, f));
-            Af[e] = sfma(-sc.wt2, X, sfma(-sc.kf, dd, f));
-          } else if (STAGE == kStage4) {
-            // the D3 terms of A4 and A_fin, left by stage 3 in D
-            const S d3 = Dn[e];
-            R = sfma(-sc.at43, X, sfma(-sc.a43e3, d3, A4[e]));
-            A4[e] = R;
-            Af[e] = sfma(-sc.wt3, X, sfma(-sc.w3e3, d3, Af[e]));
-          } else {  // kFinal: F^{n+1}, with the D4 term left by stage 4 in D
-            R = sfma(-sc.wt4, X, sfma(-sc.w4e4, Dn[e], Af[e]));
-            F[e] = R;
-          }
-          accumulate<DIM, QP, QC>(p, mom[k], pop, R);
+    for (int j = 0; j < W; ++j)
+      if (j < nq) {
+        const int64_t o = (p0 + j) * N;
+        const double R = cur[j];
+        if constexpr (DIM == 1 && STAGE != kStage3 && STAGE != kStage4) {
+          const double fe = __dmul_rn(h[j], f), D = __dsub_rn(R, fe);
+          (Dn + o)[c] = D;
+          (Fout + o)[c] = fma(sc.c2, D, fe);
+        } else {
+          const double D = fma(-h[j], f, R);
+          (Dn + o)[c] = D;
+          (Fout + o)[c] = fma(-kd, D, R);
         }
       }
-    }
-    __syncthreads();  // every thread past its last use of hx, hy
-  }
-
-  // ---- pass 2: equilibrium of the moments and closed-form relaxation
+  };
+  auto load_row = [&](int p0, int nq) {
 #pragma unroll
-  for (int k = 0; k < CPT; ++k) {
-    if (!valid[k]) continue;
-    double n, ux, uy, T;
-    if (!moments_to_nut<DIM>(geo.invDK, to_fp64(mom[k]), n, ux, uy, T)) {
-      atomicOr(p.status, 1u);
-      if (geo.prob >= 0) atomicOr(&p.pstatus[geo.prob], 1u);
-    }
-    EqCell<DIM, QP, QC> eq64;
-    make_eq_nut<DIM, QP, QC>(p, geo.kchi, n, ux, uy, T, eq64);
-    EqCellS<DIM, QP, QC, S> eq;
-    to_storage(eq64, eq);
-    const int64_t c = cell[k];
+    for (int j = 0; j < W; ++j)
+      if (j < nq) nxt[j] = (Rin + (p0 + j) * N)[c];
+  };
+  auto take_row = [&]() {
 #pragma unroll
-    for (int pop = 0; pop < L::P; ++pop) {
-      const int64_t e = pop * N + c;
-      const S fe = feq_of<DIM, QP, QC, S>(eq, pop);
-      if (STAGE == kStage3) {
-        // F3 relaxed; D3 goes to D (free until the final stage rewrites it),
-        // and stage 4 applies its terms to A4 and A_fin as it reads them
-        const S R = F3[e];
-        const S D3 = R - fe;
-        F3[e] = sfma(-sc.a33e3, D3, R);
-        Dn[e] = D3;
-      } else if (STAGE == kStage4) {
-        // F4 relaxed; D4 goes to D for the final stage's A_fin
-        const S R = A4[e];
-        const S D4 = R - fe;
-        A4[e] = sfma(-sc.a44e4, D4, R);
-        Dn[e] = D4;
-      } else {  // kPrep / kFinal: D and F2 of the new state
-        const S f = F[e];
-        const S dd = f - fe;
-        Dn[e] = dd;
-        F2[e] = sfma(sc.c2, dd, fe);
-      }
+    for (int j = 0; j < W; ++j) cur[j] = nxt[j];
+  };
+  double h[QP];
+  axis_g<QP>(p.wHp, ux, T, h);
+  if constexpr (DIM == 1) {
+    load_row(QP, QC);
+    relax_row(0, QP, h, n);
+    take_row();
+    const double nchi = geo.kchi * T * n;
+    if constexpr (QC == QP) {
+      relax_row(QP, QC, h, nchi);
+    } else {
+      double hc[QC];
+      axis_g<QC>(p.wHc, ux, T, hc);
+      relax_row(QP, QC, hc, nchi);
+    }
+  } else {
+    const double kT = geo.kchi * T;
+    {
+      double gy[QP];
+      axis_g<QP>(p.wHp, uy, T, gy);
+#pragma unroll
+      for (int j = 0; j < QP; ++j) fac[j * FS] = n * gy[j];
+    }
+    if constexpr (QC != QP) {
+      double gy[QC];
+      axis_g<QC>(p.wHc, uy, T, gy);
+#pragma unroll
+      for (int j = 0; j < QC; ++j) fac[(QP + j) * FS] = kT * n * gy[j];
+    }
+#pragma unroll 1
+    for (int r = 0; r < QP; ++r) {
+      if (r + 1 < QP) load_row((r + 1) * QP, QP);
+      else load_row(QP * QP, QC);
+      relax_row(r * QP, QP, h, fac[r * FS]);
+      take_row();
+    }
+    double hc[QC];
+    if constexpr (QC != QP) axis_g<QC>(p.wHc, ux, T, hc);
+#pragma unroll 1
+    for (int r = 0; r < QC; ++r) {
+      if (r + 1 < QC) load_row(QP * QP + (r + 1) * QC, QC);
+      if constexpr (QC == QP) relax_row(QP * QP + r * QC, QC, h, kT * fac[r * FS]);
+      else relax_row(QP * QP + r * QC, QC, hc, fac[(QP + r) * FS]);
+      take_row();
     }
   }
 }
 
-// One tile per CTA, the grid covering one problem.
-template <int DIM, int QP, int QC, int STAGE, typename S, int VAR = 0>
-__global__ void __launch_bounds__(TileCfg<DIM, VAR>::NT)
-    stage_kernel(const __grid_constant__ DevParams p) {
-  __shared__ TileSmem<DIM, S, VAR> sm;
+// ---- explicit part of one population of a cell -----------------------------
+
+// The inputs of the update: stage 3 F and D; stage 4 A4, D (holding D3) and
+// A_fin; final A_fin and D (holding D4).
+struct UpdateIn {
+  double a, d, b;
+};
+template <int STAGE>
+__device__ __forceinline__ UpdateIn load_update(const DevParams& p, int64_t o, unsigned c) {
+  UpdateIn u;
+  u.a = ((const double*)(STAGE == kStage3 ? p.F : STAGE == kStage4 ? p.A4 : p.Af) + o)[c];
+  u.d = ((const double*)p.D + o)[c];
+  u.b = STAGE == kStage4 ? ((const double*)p.Af + o)[c] : 0.0;
+  return u;
+}
+// R_i of the stage, and the running accumulators to memory.
+// PARK: R too, for a second pass of the cell's owner; the final stage's R is the
+// new state.
+template <int STAGE, bool PARK = true>
+__device__ __forceinline__ double store_update(const DevParams& p, int64_t o, unsigned c, bool valid,
+                                               const UpdateIn& u, double X) {
+  const StageCoef& sc = p.sc;
+  double R;
+  if constexpr (STAGE == kStage3) {
+    R = fma(-sc.at32, X, fma(-sc.k3, u.d, u.a));
+    const double a4 = fma(-sc.at42, X, fma(-sc.k4, u.d, u.a));
+    const double af = fma(-sc.wt2, X, fma(-sc.kf, u.d, u.a));
+    if (valid) {
+      if (PARK) ((double*)p.F3 + o)[c] = R;
+      ((double*)p.A4 + o)[c] = a4;
+      ((double*)p.Af + o)[c] = af;
+    }
+  } else if constexpr (STAGE == kStage4) {
+    R = fma(-sc.at43, X, fma(-sc.a43e3, u.d, u.a));
+    const double af = fma(-sc.wt3, X, fma(-sc.w3e3, u.d, u.b));
+    if (valid) {
+      if (PARK) ((double*)p.A4 + o)[c] = R;
+      ((double*)p.Af + o)[c] = af;
+    }
+  } else {  // kFinal: F^{n+1}
+    R = fma(-sc.wt4, X, fma(-sc.w4e4, u.d, u.a));
+    if (valid) ((double*)p.F + o)[c] = R;
+  }
+  return R;
+}
+
+// ---- 2-D ------------------------------------------------------------------------
+
+// Moment sums of a cell over groups of 4 populations.  On the lattice of
+// 8 x 8 momenta the groups run along kx, first all ky of kx = 0..3, then of
+// kx = 4..7: row sums feed jy and the y part of e, and the four column sums
+// feed n, jx and the x part of e once per half, 9 binary64 operations per
+// group instead of 16.
+constexpr int kG = 4;  // populations per group
+template <int QP, int QC>
+struct GroupMoments {
+  static constexpr bool kHalves = QP == 8;
+  static constexpr int P = Lat<2, QP, QC>::P;
+  static constexpr int NG = (P + kG - 1) / kG;
+  Moments m;
+  double col[kHalves ? 4 : 1];
+  // first population of the gi-th group
+  __device__ static __forceinline__ int first(int gi) {
+    if constexpr (kHalves) return gi < 8 ? gi * 8 : gi < 16 ? gi * 8 - 60 : gi * 4;
+    else return gi * kG;
+  }
+  __device__ __forceinline__ void add(const DevParams& p, int g0, const double (&v)[kG]) {
+    if constexpr (kHalves) {
+      const double r = (v[0] + v[1]) + (v[2] + v[3]);
+      if (g0 < 64) {
+        m.jy = fma(p.py[g0], r, m.jy);
+        m.e = fma(p.pp2[g0 >> 3], r, m.e);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) col[g] += v[g];
+      } else {
+        m.e += r;
+      }
+    } else {
+#pragma unroll
+      for (int g = 0; g < kG; ++g)
+        if (g0 + g < P) accumulate<2, QP, QC>(p, m, g0 + g, v[g]);
+    }
+  }
+  // after group gi: fold the columns of a finished half
+  __device__ __forceinline__ void fold(const DevParams& p, int gi) {
+    if constexpr (kHalves) {
+      if (gi == 7 || gi == 15) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const int k = gi == 7 ? g : g + 4;
+          m.n += col[g];
+          m.jx = fma(p.pp[k], col[g], m.jx);
+          m.e = fma(p.pp2[k], col[g], m.e);
+          col[g] = 0.0;
+        }
+      }
+    }
+  }
+};
+
+// Named barriers of the two roles of a 2-D CTA.
+__device__ __forceinline__ void bar_sync(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+// Tile of 16 x 16 cells; 256 marching and 256 updating threads.
+struct Tile2 {
+  static constexpr int TX = 16, TY = 16, NM = 256, NU = 256, SEG = 8;
+  static constexpr int SX = TX + 2 * H + 1, SY = TY + 2 * H;  // padded row pitch
+};
+template <int QP, int QC>
+struct Smem2 {
+  static constexpr int P = Lat<2, QP, QC>::P;
+  int64_t tile[2][kG][Tile2::SY][Tile2::SX];  // cells + halo: binary64, then integers
+  // flux differences along x and y, in units of the scale with exponent ex
+  // (0: binary64 bits)
+  int64_t hx[2][kG][Tile2::TY][Tile2::TX + 1];
+  int64_t hy[2][kG][Tile2::TX][Tile2::TY + 1];
+  double fac[QP + (QC == QP ? 0 : QC)][Tile2::NU];
+  AdvCoef coef[P];  // dt |p| / ds
+  int cex[P];
+  int ex[2][kG];
+  int mx[2][kG];    // largest magnitude words of the group's tiles
+};
+
+// One fused stage.  Integer and binary64 work run side by side: 8 warps march
+// (staging, scaling and the fixed-point MP-9 flux differences: integer pipes)
+// one group of populations ahead of 8 warps that update (explicit parts,
+// moments and, per tile, pass 2: binary64 pipe), through two buffers of flux
+// differences.  The CTAs walk the tiles, so the march of the next tile runs
+// during pass 2.
+// Measured at 512 x 512 x 128 populations, per step: 9.93 ms with the march in
+// binary64 (that pipe 78 % busy), 3.64 ms with every warp marching and
+// updating in turn (the pipes idle in turn), 3.29 ms so.  What bounds it now:
+// about 680 instructions per population-cell and stage at half the issue
+// rate, the integer pipe and the binary64 pipe each about half busy; 16 warps
+// a CTA wait on the fixed latency of 64-bit integer chains.
+template <int QP, int QC, int STAGE, int CTAS>
+__global__ void __launch_bounds__(Tile2::NM + Tile2::NU, CTAS)
+    stage_kernel_2d(const __grid_constant__ DevParams p, int ntx, int ntiles) {
+  using L = Lat<2, QP, QC>;
+  using GM = GroupMoments<QP, QC>;
+  using T2 = Tile2;
+  constexpr int TX = T2::TX, TY = T2::TY, NM = T2::NM, NU = T2::NU;
+  constexpr int kMarchBar = 1, kFull = 2, kEmpty = 4;  // + buffer
+  extern __shared__ __align__(16) unsigned char smraw[];
+  auto& sm = *reinterpret_cast<Smem2<QP, QC>*>(smraw);
+  const int64_t N = p.N;
+  const int items = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x * GM::NG;
+  for (int pop = threadIdx.x; pop < L::P; pop += NM + NU)
+    sm.coef[pop] = advection_coef(p.cx[pop], p.cy[pop], sm.cex[pop]);
+  if (threadIdx.x < 2 * kG) sm.mx[threadIdx.x / kG][threadIdx.x % kG] = 0;
+  __syncthreads();
+
+  if (threadIdx.x < NM) {
+    // ---- march
+    const int tid = threadIdx.x;
+    const double* __restrict__ const adv =
+        (const double*)(STAGE == kStage3 ? p.F2 : STAGE == kStage4 ? p.F3 : p.A4);
+    // the thread's half line: population tg of the group; one warp takes the
+    // x lines of a population, the next its y lines (16 lines a half-warp
+    // keep the 8-byte accesses free of bank conflicts)
+    const int tg = tid / 64, ln = tid % 16, s0 = (tid / 16 % 2) * T2::SEG;
+    const bool xline = (tid & 32) == 0;
+    // the thread's staged cells (staged_pos skips the corners): ghosts by
+    // index clamp or wrap
+    constexpr int NST = TY * (TX + 2 * H) + 2 * H * TX;
+    constexpr int J = (NST + NM - 1) / NM;
+    int soff[J], goff[J];
+    bool has[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      int r, c;
+      staged_pos(tid + j * NM, 2, TX, TY, r, c);
+      has[j] = tid + j * NM < NST;
+      soff[j] = r * T2::SX + c;
+    }
+    auto set_tile = [&](int t) {
+      const int x0 = t % ntx * TX, y0 = t / ntx * TY;
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        int r, c;
+        staged_pos(tid + j * NM, 2, TX, TY, r, c);
+        goff[j] = wrap_or_clamp(y0 - H + r, p.ny, p.bc) * p.nx + wrap_or_clamp(x0 - H + c, p.nx, p.bc);
+      }
+    };
+    auto prefetch = [&](int b, int g0) {
+#pragma unroll
+      for (int g = 0; g < kG; ++g)
+        if (g0 + g < L::P) {
+          const double* __restrict__ src = adv + (g0 + g) * N;
+#pragma unroll
+          for (int j = 0; j < J; ++j)
+            if (has[j]) cp_async((double*)&sm.tile[b][g][0][0] + soff[j], src + (unsigned)goff[j]);
+        }
+      cp_async_commit();
+    };
+    int tile = blockIdx.x, gi = 0;
+    set_tile(tile);
+    prefetch(0, GM::first(0));
+    for (int it = 0; it < items; ++it) {
+      const int b = it & 1, g0 = GM::first(gi);
+      // the scale of each population's tile: the largest magnitude
+      cp_async_wait_all();
+#pragma unroll
+      for (int g = 0; g < kG; ++g) {
+        int m = 0;
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+          if (has[j]) m = max(m, mag_word(dfrom((&sm.tile[b][g][0][0])[soff[j]])));
+        m = (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
+        if (tid % 32 == g) atomicMax(&sm.mx[b][g], m);
+      }
+      bar_sync(kMarchBar, NM);  // the magnitudes are in; the previous march is done
+      int ngi = gi + 1;
+      if (ngi == GM::NG) {
+        ngi = 0;
+        tile += gridDim.x;
+        if (it + 1 < items) set_tile(tile);
+      }
+      if (it + 1 < items) prefetch(b ^ 1, GM::first(ngi));
+      if (tid < kG) sm.mx[b ^ 1][tid] = 0;
+      // cells to integers, once each and by the thread that copied them
+#pragma unroll
+      for (int g = 0; g < kG; ++g) {
+        const int emax = sm.mx[b][g] >> 20;
+        if (emax >= kQExpMin && emax <= kQExpMax) {
+#pragma unroll
+          for (int j = 0; j < J; ++j)
+            if (has[j]) {
+              int64_t& v = (&sm.tile[b][g][0][0])[soff[j]];
+              v = q_of(dfrom(v), emax);
+            }
+        }
+      }
+      bar_sync(kMarchBar, NM);  // the group's tile is in
+      if (it >= 2) bar_sync(kEmpty + b, NM + NU);  // the update is done with this buffer
+      const int pop = g0 + tg;
+      const double pv = pop < L::P ? (xline ? p.px[pop] : p.py[pop]) : 0.0;
+      const int sgn = pv >= 0.0 ? 1 : -1;
+      const int first = sgn > 0 ? s0 : s0 + T2::SEG - 1;
+      const int step = xline ? 1 : T2::SX;
+      const int64_t* line = xline ? &sm.tile[b][tg][ln + H][H] : &sm.tile[b][tg][H][ln + H];
+      const int64_t* up = line + (first - sgn) * step;
+      int64_t* out = xline ? &sm.hx[b][tg][ln][first] : &sm.hy[b][tg][ln][first];
+      const int emax = sm.mx[b][tg] >> 20;
+      const bool fixed = emax >= kQExpMin && emax <= kQExpMax;
+      if (tid % 64 == 0) sm.ex[b][tg] = fixed ? emax : 0;
+      if (pop < L::P) {
+        if (fixed) mp9_march_delta_int<T2::SEG>(up, sgn * step, out, sgn);
+        else mp9_march_delta_fp64((const double*)up, sgn * step, out, sgn, T2::SEG);
+      }
+      bar_arrive(kFull + b, NM + NU);
+      gi = ngi;
+    }
+  } else {
+    // ---- update
+    const int tid = threadIdx.x - NM;
+    const int lx = tid % TX, ly = tid / TX;
+    const Geo geo{p.nx, p.ny, 0, p.kchi, p.invDK, p.dtdx, p.dtdy, -1};
+    int it = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      const int x = tile % ntx * TX + lx, y = tile / ntx * TY + ly;
+      const bool valid = x < p.nx && y < p.ny;
+      // (a thread without a cell reads the first one and stores nothing)
+      const unsigned c = valid ? (unsigned)y * p.nx + x : 0u;
+      GM mom = {};
+      UpdateIn in[kG];
+      auto load = [&](int g0, UpdateIn (&u)[kG]) {
+#pragma unroll
+        for (int g = 0; g < kG; ++g)
+          if (g0 + g < L::P) u[g] = load_update<STAGE>(p, (g0 + g) * N, c);
+      };
+      for (int gi = 0; gi < GM::NG; ++gi, ++it) {
+        const int b = it & 1, g0 = GM::first(gi);
+        load(g0, in);
+        bar_sync(kFull + b, NM + NU);  // the group's flux differences are in
+        double R[kG];
+#pragma unroll
+        for (int g = 0; g < kG; ++g) {
+          const int pop = g0 + g;
+          R[g] = 0.0;
+          if (pop < L::P) {
+            // X = dt p . grad F
+            const int64_t dx = sm.hx[b][g][ly][lx], dy = sm.hy[b][g][lx][ly];
+            const int ex = sm.ex[b][g];
+            double X = q_to_double(advection_int(sm.coef[pop], dx, dy), ex + sm.cex[pop]);
+            if (!ex) X = advection_bits(p.cx[pop], p.cy[pop], dx, dy);
+            R[g] = store_update<STAGE>(p, pop * N, c, valid, in[g], X);
+          }
+        }
+        if (it + 2 < items) bar_arrive(kEmpty + b, NM + NU);
+        mom.add(p, g0, R);
+        mom.fold(p, gi);
+      }
+      if (valid) relax_cell64<2, QP, QC, STAGE, NU>(p, geo, c, mom.m, &sm.fac[0][tid]);
+    }
+  }
+}
+
+// ---- 1-D ------------------------------------------------------------------------
+//
+// 1-D problems march in binary64 (fdlb_mp9.cuh): batches, single problems and
+// the checkpointed runs of the adjoint agree bit for bit, and the adjoint
+// recomputes the limiter's choices with the march's own comparisons.
+
+// Tile shapes: cells, threads, populations per group and interfaces per march
+// task (a tile of TX cells has TX + 1 interfaces).
+template <int VAR>
+struct Tile1;
+template <>
+struct Tile1<0> {
+  static constexpr int TX = 127, NT = 128, G = 8, SEG = 8;
+};
+template <>
+struct Tile1<1> {
+  static constexpr int TX = 63, NT = 128, G = 16, SEG = 8;
+};
+template <>
+struct Tile1<2> {
+  static constexpr int TX = 255, NT = 128, G = 8, SEG = 16;
+};
+// short single problems, so that their tiles still spread over the SMs
+template <>
+struct Tile1<3> {
+  static constexpr int TX = 15, NT = 64, G = 16, SEG = 4;
+};
+template <>
+struct Tile1<4> {
+  static constexpr int TX = 31, NT = 64, G = 16, SEG = 8;
+};
+
+// Shared memory of one tile: the advected populations of a group on tile +
+// halo, and the interface values.
+template <int VAR>
+struct Smem1 {
+  using C = Tile1<VAR>;
+  double tile[C::G][C::TX + 2 * H];
+  double hx[C::G][C::TX + 1];
+};
+
+// One tile (first cell x0 of the problem of geo) of one fused stage.  Ends
+// with every thread past its last use of the shared memory, so a persistent
+// CTA may start its next tile at once.
+template <int QP, int QC, int STAGE, int VAR>
+__device__ __forceinline__ void stage_tile_1d(const DevParams& p, const Geo& geo, int x0, Smem1<VAR>& sm) {
+  using C = Tile1<VAR>;
+  constexpr int P = QP + QC;
+  constexpr int TX = C::TX, NT = C::NT, G = C::G, SEG = C::SEG, NSEG = (TX + 1) / SEG;
+  constexpr int CPT = (TX + NT - 1) / NT;
+  static_assert(NSEG * SEG == TX + 1 && G * NSEG == NT, "one march task per thread");
+  const int tid = threadIdx.x;
+  const int64_t N = p.N;
+  // the thread's cells (a slot without one reads the problem's first cell and
+  // stores nothing)
+  int lxs[CPT];
+  unsigned cell[CPT];
+  bool valid[CPT];
+  Moments mom[CPT];
+#pragma unroll
+  for (int k = 0; k < CPT; ++k) {
+    const int ci = tid + k * NT;
+    lxs[k] = ci < TX ? ci : 0;
+    valid[k] = ci < TX && x0 + ci < geo.nx;
+    cell[k] = (unsigned)geo.base + (valid[k] ? x0 + ci : 0);
+    mom[k] = {};
+  }
+  const double* __restrict__ const adv =
+      (const double*)(STAGE == kStage3 ? p.F2 : STAGE == kStage4 ? p.F3 : p.A4);
+  const int tg = tid / NSEG;  // the march task's population in a group
+  // the thread's staged cells: ghosts by index clamp or wrap
+  constexpr int NST = TX + 2 * H;
+  constexpr int J = (NST + NT - 1) / NT;
+  int goff[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    const int e = tid + j * NT;
+    goff[j] = e < NST ? wrap_or_clamp(x0 - H + e, geo.nx, p.bc) : -1;
+  }
+  // the group's advected populations, copied asynchronously; the next group's
+  // copies run during this group's update
+  auto prefetch = [&](int g0) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      if (g0 + g >= P) break;
+      const double* __restrict__ src = adv + ((g0 + g) * N + geo.base);
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+        if (goff[j] >= 0) cp_async(&sm.tile[g][tid + j * NT], src + (unsigned)goff[j]);
+    }
+    cp_async_commit();
+  };
+  prefetch(0);
+  for (int g0 = 0; g0 < P; g0 += G) {
+    cp_async_wait_all();
+    __syncthreads();  // the group's tile is in; the previous update is done
+    // every interface value once, marching upwind -> downwind
+    if (g0 + tg < P) {
+      const int sgn = p.px[g0 + tg] >= 0.0 ? 1 : -1;
+      const MarchTask t = march_task(tid, 1, TX, 1, SEG, NST, sgn);
+      mp9_march_fp64<SEG>(&sm.tile[tg][t.bc_], sgn, &sm.hx[tg][t.ofirst], sgn);
+    }
+    // the own cells' inputs, in flight across the barrier
+    UpdateIn in[CPT][G];
+#pragma unroll
+    for (int k = 0; k < CPT; ++k)
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+        if (g0 + g < P) in[k][g] = load_update<STAGE>(p, (g0 + g) * N, cell[k]);
+    __syncthreads();  // the march is done with the tile
+    if (g0 + G < P) prefetch(g0 + G);
+#pragma unroll
+    for (int k = 0; k < CPT; ++k)
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int pop = g0 + g;
+        if (pop >= P) break;
+        // X = dt p dF/dx (single problems use the host's dt p/dx, the same
+        // product)
+        const double cx = geo.prob < 0 ? p.cx[pop] : geo.dtdx * p.px[pop];
+        const double X = cx * (sm.hx[g][lxs[k] + 1] - sm.hx[g][lxs[k]]);
+        const double R = store_update<STAGE>(p, pop * N, cell[k], valid[k], in[k][g], X);
+        accumulate<1, QP, QC>(p, mom[k], pop, R);
+      }
+  }
+  __syncthreads();  // every thread past its last use of hx
+#pragma unroll
+  for (int k = 0; k < CPT; ++k)
+    if (valid[k]) relax_cell64<1, QP, QC, STAGE, 1>(p, geo, cell[k], mom[k], nullptr);
+}
+
+// One tile per CTA, the grid covering one problem (at most 128 registers: 4
+// CTAs per SM keep the binary64 pipe about 75 % busy).
+template <int QP, int QC, int STAGE, int VAR>
+__global__ void __launch_bounds__(Tile1<VAR>::NT, 4) stage_kernel(const __grid_constant__ DevParams p) {
+  __shared__ Smem1<VAR> sm;
   const Geo geo{p.nx, p.ny, 0, p.kchi, p.invDK, p.dtdx, p.dtdy, -1};
-  stage_tile<DIM, QP, QC, STAGE, S, VAR>(p, geo, blockIdx.x * TileCfg<DIM, VAR>::TX,
-                                         blockIdx.y * TileCfg<DIM, VAR>::TY, sm);
+  stage_tile_1d<QP, QC, STAGE, VAR>(p, geo, blockIdx.x * Tile1<VAR>::TX, sm);
 }
 
 // Batches of 1-D problems: a persistent grid walks the tile work list of all
 // problems (each tile within one problem, ghosts clamped at its own ends).
-template <int QP, int QC, int STAGE, typename S, int VAR>
-__global__ void __launch_bounds__(TileCfg<1, VAR>::NT)
-    batch_stage_kernel(const __grid_constant__ DevParams p) {
-  __shared__ TileSmem<1, S, VAR> sm;
+template <int QP, int QC, int STAGE, int VAR>
+__global__ void __launch_bounds__(Tile1<VAR>::NT, 4) batch_stage_kernel(const __grid_constant__ DevParams p) {
+  __shared__ Smem1<VAR> sm;
   for (int w = blockIdx.x; w < p.nwork; w += gridDim.x) {
     const WorkItem it = p.work[w];
     const BatchProblem& bp = p.probs[it.prob];
     const Geo geo{bp.nx, 1, bp.base, bp.kchi, bp.invDK, bp.dtdx, 0.0, it.prob};
-    stage_tile<1, QP, QC, STAGE, S, VAR>(p, geo, it.x0, 0, sm);
+    stage_tile_1d<QP, QC, STAGE, VAR>(p, geo, it.x0, sm);
   }
 }
 
@@ -272,6 +615,25 @@ __device__ __forceinline__ int find_problem(const DevParams& p, int64_t c) {
     else hi = mid - 1;
   }
   return lo;
+}
+
+// D and F2 of a state that was set (fdlb_init_riemann, fdlb_set_state), one
+// cell per thread.
+template <int DIM, int QP, int QC>
+__global__ void __launch_bounds__(128) prep_kernel(const __grid_constant__ DevParams p) {
+  __shared__ double fac[DIM == 2 ? QP + QC : 1][128];
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= p.N) return;
+  Geo geo{p.nx, p.ny, 0, p.kchi, p.invDK, p.dtdx, p.dtdy, -1};
+  if (p.nprob > 0) {
+    geo.prob = find_problem(p, c);
+    geo.kchi = p.probs[geo.prob].kchi;
+    geo.invDK = p.probs[geo.prob].invDK;
+  }
+  Moments m = {};
+  for (int pop = 0; pop < Lat<DIM, QP, QC>::P; ++pop)
+    accumulate<DIM, QP, QC>(p, m, pop, ((const double*)p.F + pop * p.N)[c]);
+  relax_cell64<DIM, QP, QC, kPrep, 128>(p, geo, (unsigned)c, m, &fac[0][threadIdx.x]);
 }
 
 template <int QP, int QC, typename S>
@@ -403,38 +765,73 @@ __global__ void moments_adjoint_kernel(const __grid_constant__ DevParams p,
   }
 }
 
-template <int DIM, int QP, int QC, typename S, int VAR>
-int launch_stage_tsv(const DevParams& p, int stage, cudaStream_t s) {
-  using C = TileCfg<DIM, VAR>;
-  dim3 grid((p.nx + C::TX - 1) / C::TX, DIM == 2 ? (p.ny + C::TY - 1) / C::TY : 1);
+template <int DIM, int QP, int QC>
+int launch_prep(const DevParams& p, cudaStream_t s) {
+  prep_kernel<DIM, QP, QC><<<(unsigned)((p.N + 127) / 128), 128, 0, s>>>(p);
+  return (int)cudaGetLastError();
+}
+
+template <int QP, int QC, int STAGE, int CTAS>
+int launch_stage_2d_c(const DevParams& p, int ntx, int ntiles, int nsm, cudaStream_t s) {
+  constexpr int bytes = (int)sizeof(Smem2<QP, QC>);
+  const cudaError_t e = cudaFuncSetAttribute(stage_kernel_2d<QP, QC, STAGE, CTAS>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return (int)e;
+  const int grid = ntiles < CTAS * nsm ? ntiles : CTAS * nsm;
+  stage_kernel_2d<QP, QC, STAGE, CTAS><<<grid, Tile2::NM + Tile2::NU, bytes, s>>>(p, ntx, ntiles);
+  return (int)cudaGetLastError();
+}
+
+// Grids of no more tiles than SMs run one CTA per SM, whose threads then have
+// 128 registers; larger ones run two of 64 (some spills, twice the warps):
+// 96 x 70, 30 tiles, 0.165 against 0.178 ms a stage; 512 x 512, 1024 tiles,
+// 1.21 against 1.10.
+template <int QP, int QC, int STAGE>
+int launch_stage_2d(const DevParams& p, cudaStream_t s) {
+  const int ntx = (p.nx + Tile2::TX - 1) / Tile2::TX, nty = (p.ny + Tile2::TY - 1) / Tile2::TY;
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return (int)e;
+  const int ntiles = ntx * nty;
+  return ntiles <= nsm ? launch_stage_2d_c<QP, QC, STAGE, 1>(p, ntx, ntiles, nsm, s)
+                       : launch_stage_2d_c<QP, QC, STAGE, 2>(p, ntx, ntiles, nsm, s);
+}
+
+template <int QP, int QC, int VAR>
+int launch_stage_1d(const DevParams& p, int stage, cudaStream_t s) {
+  using C = Tile1<VAR>;
+  const int grid = (p.nx + C::TX - 1) / C::TX;
   switch (stage) {
-    case kPrep: stage_kernel<DIM, QP, QC, kPrep, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
-    case kStage3: stage_kernel<DIM, QP, QC, kStage3, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
-    case kStage4: stage_kernel<DIM, QP, QC, kStage4, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
-    default: stage_kernel<DIM, QP, QC, kFinal, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
+    case kStage3: stage_kernel<QP, QC, kStage3, VAR><<<grid, C::NT, 0, s>>>(p); break;
+    case kStage4: stage_kernel<QP, QC, kStage4, VAR><<<grid, C::NT, 0, s>>>(p); break;
+    default: stage_kernel<QP, QC, kFinal, VAR><<<grid, C::NT, 0, s>>>(p); break;
   }
   return (int)cudaGetLastError();
 }
 
-// 1-D problems pick their tile shape by length (single_1d_variant).
-template <int DIM, int QP, int QC, typename S>
-int launch_stage_ts(const DevParams& p, int stage, cudaStream_t s) {
+template <int DIM, int QP, int QC>
+int launch_stage_fp64(const DevParams& p, int stage, cudaStream_t s) {
   if constexpr (DIM == 1) {
-    switch (single_1d_variant(p.nx)) {
-      case 1: return launch_stage_tsv<1, QP, QC, S, 1>(p, stage, s);
-      case 3: return launch_stage_tsv<1, QP, QC, S, 3>(p, stage, s);
-      case 4: return launch_stage_tsv<1, QP, QC, S, 4>(p, stage, s);
-      default: return launch_stage_tsv<1, QP, QC, S, 0>(p, stage, s);
-    }
+    if (stage == kPrep) return launch_prep<1, QP, QC>(p, s);
+    // longer problems: the largest tile that still gives about one per SM
+    if (p.nx >= 127 * 152) return launch_stage_1d<QP, QC, 0>(p, stage, s);
+    if (p.nx >= 63 * 152) return launch_stage_1d<QP, QC, 1>(p, stage, s);
+    if (p.nx >= 31 * 152) return launch_stage_1d<QP, QC, 4>(p, stage, s);
+    return launch_stage_1d<QP, QC, 3>(p, stage, s);
+  } else {
+    if (stage == kPrep) return launch_prep<DIM, QP, QC>(p, s);
+    return stage == kStage3   ? launch_stage_2d<QP, QC, kStage3>(p, s)
+           : stage == kStage4 ? launch_stage_2d<QP, QC, kStage4>(p, s)
+                              : launch_stage_2d<QP, QC, kFinal>(p, s);
   }
-  return launch_stage_tsv<DIM, QP, QC, S, 0>(p, stage, s);
 }
 
 template <int DIM, int QP, int QC>
 int launch_stage_t(const DevParams& p, int stage, cudaStream_t s) {
-  // binary32 contexts run the single-pass kernels of fdlb_mixed.cu
+  // binary32 contexts run the kernels of fdlb_mixed.cu
   return p.precision == 1 ? launch_mixed_stage(p, stage, s)
-                          : launch_stage_ts<DIM, QP, QC, double>(p, stage, s);
+                          : launch_stage_fp64<DIM, QP, QC>(p, stage, s);
 }
 
 template <int DIM, int QP, int QC>
@@ -456,32 +853,32 @@ int launch_moments_t(const DevParams& p, double* n, double* ux, double* uy, doub
   return (int)cudaGetLastError();
 }
 
-template <int QP, int QC, typename S, int VAR>
+template <int QP, int QC, int VAR>
 int launch_batch_stage_v(const DevParams& p, int stage, cudaStream_t s) {
-  using C = TileCfg<1, VAR>;
+  using C = Tile1<VAR>;
   const int grid = p.bgrid > 0 ? p.bgrid : 1;
   switch (stage) {
-    case kPrep: batch_stage_kernel<QP, QC, kPrep, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
-    case kStage3: batch_stage_kernel<QP, QC, kStage3, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
-    case kStage4: batch_stage_kernel<QP, QC, kStage4, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
-    default: batch_stage_kernel<QP, QC, kFinal, S, VAR><<<grid, C::NT, 0, s>>>(p); break;
+    case kPrep: return launch_prep<1, QP, QC>(p, s);
+    case kStage3: batch_stage_kernel<QP, QC, kStage3, VAR><<<grid, C::NT, 0, s>>>(p); break;
+    case kStage4: batch_stage_kernel<QP, QC, kStage4, VAR><<<grid, C::NT, 0, s>>>(p); break;
+    default: batch_stage_kernel<QP, QC, kFinal, VAR><<<grid, C::NT, 0, s>>>(p); break;
   }
   return (int)cudaGetLastError();
 }
 
-template <int QP, int QC, typename S>
-int launch_batch_stage_s(const DevParams& p, int stage, cudaStream_t s) {
+template <int QP, int QC>
+int launch_batch_stage_fp64(const DevParams& p, int stage, cudaStream_t s) {
   switch (p.variant) {
-    case 1: return launch_batch_stage_v<QP, QC, S, 1>(p, stage, s);
-    case 2: return launch_batch_stage_v<QP, QC, S, 2>(p, stage, s);
-    default: return launch_batch_stage_v<QP, QC, S, 0>(p, stage, s);
+    case 1: return launch_batch_stage_v<QP, QC, 1>(p, stage, s);
+    case 2: return launch_batch_stage_v<QP, QC, 2>(p, stage, s);
+    default: return launch_batch_stage_v<QP, QC, 0>(p, stage, s);
   }
 }
 
 template <int QP, int QC>
 int launch_batch_stage_t(const DevParams& p, int stage, cudaStream_t s) {
   return p.precision == 1 ? launch_mixed_batch_stage(p, stage, s)
-                          : launch_batch_stage_s<QP, QC, double>(p, stage, s);
+                          : launch_batch_stage_fp64<QP, QC>(p, stage, s);
 }
 
 template <int QP, int QC>

@@ -455,11 +455,7 @@ template <>
 struct Tile1<2> {
   static constexpr int TX = 255, NT = 128, G = 8, SEG = 16;
 };
-// short single problems, so that their tiles still spread over the SMs
-template <>
-struct Tile1<3> {
-  static constexpr int TX = 15, NT = 64, G = 16, SEG = 4;
-};
+// single problems of middle length, so that their tiles still spread over the SMs
 template <>
 struct Tile1<4> {
   static constexpr int TX = 31, NT = 64, G = 16, SEG = 8;
@@ -571,6 +567,111 @@ __global__ void __launch_bounds__(Tile1<VAR>::NT, 4) stage_kernel(const __grid_c
   __shared__ Smem1<VAR> sm;
   const Geo geo{p.nx, p.ny, 0, p.kchi, p.invDK, p.dtdx, p.dtdy, -1};
   stage_tile_1d<QP, QC, STAGE, VAR>(p, geo, blockIdx.x * Tile1<VAR>::TX, sm);
+}
+
+// One stage (or, STAGE = kPrep, D and F2 of a state that was set) of a short
+// 1-D problem: 8 threads a population, one interface each, and the 7 cells
+// between them.  A warp's binary64 instruction takes 64 cycles whether 1 or 32
+// of its lanes work, so a short problem's time is the number of binary64
+// instructions on one thread's path; here that is one interface, one
+// population's update, QP + QC steps of the moment sums (the three sums of
+// the cells in the lanes of every warp, so that they need no second barrier)
+// and one node's equilibrium, about 100, against about 400 for a thread that
+// owns a cell.  Every value is formed by the operations of stage_tile_1d in
+// their order, so the results are the same bits.
+// Measured a step: 400 cells of 16 populations 16.4 us against 51 (tiles of 15
+// cells), of 8 populations 13.3 against 33.  Its work per cell is larger, so
+// it gives way to the tiles where the chip is full: at 65 536
+// population-cells, 43.9 us (16) and 34.8 us (8) against 46.5 and 35.7.
+constexpr int kSmallCells = 7;
+constexpr int kSmallPopCells = 65536;
+template <int QP, int QC>
+constexpr int small_threads() { return ((QP + QC) * 8 + 31) / 32 * 32; }
+template <int QP, int QC, int STAGE>
+__global__ void __launch_bounds__(small_threads<QP, QC>())
+    small_stage_kernel(const __grid_constant__ DevParams p) {
+  constexpr int P = QP + QC;
+  __shared__ double Rs[P][8];
+  const int tid = threadIdx.x, lc = tid % 8, lane = tid % 32;
+  const int pop = tid / 8 < P ? tid / 8 : P - 1;
+  const int x = blockIdx.x * kSmallCells + lc;  // cell, and the interface left of it
+  const bool valid = tid / 8 < P && lc < kSmallCells && x < p.nx;
+  const unsigned c = x < p.nx ? x : p.nx - 1;
+  const int64_t o = pop * p.N;
+  // the node's column of the equilibrium table: node k of Q, or its mirror
+  const int Q = pop < QP ? QP : QC, k = pop < QP ? pop : pop - QP;
+  const bool mirror = k >= (Q + 1) / 2;
+  constexpr int QM = QP > QC ? QP : QC;
+  double w[QM];
+#pragma unroll
+  for (int l = 0; l < QM; ++l)
+    w[l] = l < Q ? (pop < QP ? p.wHp : p.wHc)[l * kMaxQ + (mirror ? Q - 1 - k : k)] : 0.0;
+  double R;
+  if constexpr (STAGE == kPrep) {
+    R = ((const double*)p.F + o)[c];
+  } else {
+    // the interface's window in march order, from its upwind cell
+    const int sgn = p.px[pop] >= 0.0 ? 1 : -1;
+    const int up = sgn > 0 ? x - 1 : x;
+    const double* __restrict__ const adv =
+        (const double*)(STAGE == kStage3 ? p.F2 : STAGE == kStage4 ? p.F3 : p.A4) + o;
+    double v[9];
+#pragma unroll
+    for (int j = 0; j < 9; ++j) v[j] = adv[(unsigned)wrap_or_clamp(up + sgn * (j - 4), p.nx, p.bc)];
+    const UpdateIn in = load_update<STAGE>(p, o, c);
+    double f;
+    mp9_march_fp64<1>(v + 4, 1, &f, 1);
+    const double X = p.cx[pop] * (__shfl_down_sync(0xffffffffu, f, 1) - f);
+    R = store_update<STAGE, false>(p, o, c, valid, in, X);
+  }
+  Rs[pop][lc] = R;
+  __syncthreads();
+  // moment sums in population order: lanes 0-7 n, 8-15 j, 16-31 e
+  const int role = lane / 8;
+  double acc = 0.0;
+#pragma unroll
+  for (int q = 0; q < P; ++q) {
+    const double cf = q >= QP || role == 0 ? 1.0 : role == 1 ? p.px[q] : p.p2[q];
+    const double s = fma(cf, Rs[q][lc], acc);
+    if (q < QP || role >= 2) acc = s;
+  }
+  Moments m;
+  m.n = __shfl_sync(0xffffffffu, acc, lc);
+  m.jx = __shfl_sync(0xffffffffu, acc, 8 + lc);
+  m.jy = 0.0;
+  m.e = __shfl_sync(0xffffffffu, acc, 16 + lc);
+  double n, u, uy, T;
+  if (!moments_to_nut<1>(p.invDK, m, n, u, uy, T) && valid && pop == 0) atomicOr(p.status, 1u);
+  // the node's equilibrium (axis_g's operations)
+  double a[QM];
+  a[0] = 1.0;
+  a[1] = u;
+  const double tm1 = T - 1.0;
+#pragma unroll
+  for (int l = 2; l < QM; ++l) a[l] = fma(u, a[l - 1], ((double)(l - 1) * tm1) * a[l - 2]);
+  double ev = w[0], od = 0.0;
+#pragma unroll
+  for (int l = 1; l < QM; ++l) {
+    if (l & 1) od = fma(w[l], a[l], od);
+    else ev = fma(w[l], a[l], ev);
+  }
+  const double g = mirror ? ev - od : ev + od;
+  const double f = pop < QP ? n : p.kchi * T * n;
+  const StageCoef& sc = p.sc;
+  if constexpr (STAGE == kStage3 || STAGE == kStage4) {
+    const double D = fma(-g, f, R);
+    const double Fi = fma(STAGE == kStage3 ? -sc.a33e3 : -sc.a44e4, D, R);
+    if (valid) {
+      ((double*)p.D + o)[c] = D;
+      ((double*)(STAGE == kStage3 ? p.F3 : p.A4) + o)[c] = Fi;
+    }
+  } else {
+    const double fe = __dmul_rn(g, f), D = __dsub_rn(R, fe);
+    if (valid) {
+      ((double*)p.D + o)[c] = D;
+      ((double*)p.F2 + o)[c] = fma(sc.c2, D, fe);
+    }
+  }
 }
 
 // Batches of 1-D problems: a persistent grid walks the tile work list of all
@@ -810,15 +911,27 @@ int launch_stage_1d(const DevParams& p, int stage, cudaStream_t s) {
   return (int)cudaGetLastError();
 }
 
+template <int QP, int QC>
+int launch_small_1d(const DevParams& p, int stage, cudaStream_t s) {
+  const int grid = (p.nx + kSmallCells - 1) / kSmallCells, nt = small_threads<QP, QC>();
+  switch (stage) {
+    case kPrep: small_stage_kernel<QP, QC, kPrep><<<grid, nt, 0, s>>>(p); break;
+    case kStage3: small_stage_kernel<QP, QC, kStage3><<<grid, nt, 0, s>>>(p); break;
+    case kStage4: small_stage_kernel<QP, QC, kStage4><<<grid, nt, 0, s>>>(p); break;
+    default: small_stage_kernel<QP, QC, kFinal><<<grid, nt, 0, s>>>(p); break;
+  }
+  return (int)cudaGetLastError();
+}
+
 template <int DIM, int QP, int QC>
 int launch_stage_fp64(const DevParams& p, int stage, cudaStream_t s) {
   if constexpr (DIM == 1) {
+    if (p.nx <= kSmallPopCells / (QP + QC)) return launch_small_1d<QP, QC>(p, stage, s);
     if (stage == kPrep) return launch_prep<1, QP, QC>(p, s);
     // longer problems: the largest tile that still gives about one per SM
     if (p.nx >= 127 * 152) return launch_stage_1d<QP, QC, 0>(p, stage, s);
     if (p.nx >= 63 * 152) return launch_stage_1d<QP, QC, 1>(p, stage, s);
-    if (p.nx >= 31 * 152) return launch_stage_1d<QP, QC, 4>(p, stage, s);
-    return launch_stage_1d<QP, QC, 3>(p, stage, s);
+    return launch_stage_1d<QP, QC, 4>(p, stage, s);
   } else {
     if (stage == kPrep) return launch_prep<DIM, QP, QC>(p, s);
     return stage == kStage3   ? launch_stage_2d<QP, QC, kStage3>(p, s)

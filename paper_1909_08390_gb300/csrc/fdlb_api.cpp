@@ -278,21 +278,37 @@ int ensure_graph(fdlb_ctx* c) {
 
 // Device buffers of a context: FDLB_FP64, six binary64 population arrays
 // (F, F2, F3, A4, A_fin, D); FDLB_MIXED, eleven binary32 population arrays
-// (the two state buffers hi and lo, r3l, a4l, afl, dm, fa, fb, fc) and the
+// of P * NS values (the two state buffers hi and lo, r3l, a4l, afl, dm, fa, fb, fc) and the
 // per-cell mhi; then the four moment fields for host copies and the status
 // word.
 struct Layout {
   size_t arr, mom, mhi, total;
 };
 
-Layout buffer_layout(int precision, int P, int64_t N) {
+// Row pitch and population stride of a context's arrays (DevParams::pitch).
+// FDLB_MIXED 2-D grids are padded to whole tiles unless they are so thin that
+// the padding would cost more than an eighth and more than 2^18 cells.
+void set_strides(DevParams& p) {
+  p.pitch = p.nx;
+  p.padded = 0;
+  p.NS = p.N;
+  if (p.precision != FDLB_MIXED || p.d != 2) return;
+  const int64_t px = ((int64_t)p.nx + 15) / 16 * 16, py = ((int64_t)p.ny + 15) / 16 * 16;
+  if (px * py > (1 << 18) && 8 * px * py > 9 * p.N) return;
+  p.pitch = (int)px;
+  p.padded = 1;
+  p.NS = px * py;
+}
+
+// N cells of which each population takes NS in memory.
+Layout buffer_layout(int precision, int P, int64_t N, int64_t NS) {
   Layout L{};
   const size_t esize = precision == FDLB_MIXED ? sizeof(float) : sizeof(double);
-  L.arr = ((size_t)P * (size_t)N * esize + 255) / 256 * 256;
+  L.arr = ((size_t)P * (size_t)NS * esize + 255) / 256 * 256;
   const size_t narr = precision == FDLB_MIXED ? 11 : 6;
   L.mom = narr * L.arr;
   L.mhi = L.mom + 4 * (size_t)N * sizeof(double) + 256;
-  L.total = L.mhi + (precision == FDLB_MIXED ? 4 * (size_t)N * sizeof(double) : 0);
+  L.total = L.mhi + (precision == FDLB_MIXED ? 4 * (size_t)NS * sizeof(double) : 0);
   return L;
 }
 
@@ -323,6 +339,13 @@ void assign_buffers(fdlb_ctx* c, const Layout& L) {
   }
   c->mom = (double*)(b + L.mom);
   p.status = (unsigned*)(b + L.mom + 4 * (size_t)p.N * sizeof(double));
+}
+
+// The mixed state to (out) or from the binary64 array x of P * N values.
+int exchange_state(const fdlb_ctx* c, double* x, bool out) {
+  DevParams q = c->dp;
+  q.xstate = x;
+  return fdlb::launch_stage(q, out ? fdlb::kStateOut : fdlb::kStateIn, c->stream);
 }
 
 // A binary64 scratch array of P * N values for moving a FDLB_MIXED state to
@@ -571,7 +594,8 @@ int fdlb_create(const fdlb_grid* grid, int Qphi, int Qchi, double gamma, double 
     return cuda_err(nullptr, e, "cudaGetDevice");
   }
   p.precision = precision;
-  const Layout lay = buffer_layout(precision, p.P, N);
+  set_strides(p);
+  const Layout lay = buffer_layout(precision, p.P, N, p.NS);
   c->buf_bytes = lay.total;
   e = cudaMalloc(&c->buf, c->buf_bytes);
   if (e != cudaSuccess) {
@@ -735,8 +759,7 @@ int fdlb_get_state(fdlb_ctx* c, void* dst, int on_device) {
   if (c->precision == FDLB_MIXED) {
     // the exact binary64 value hi + lo of every population
     double* dev = on_device ? (double*)dst : mixed_exchange_buffer(c);
-    const int64_t n = (int64_t)c->dp.P * c->dp.N;
-    int le = fdlb::launch_pair_to_double(c->dp.sh, c->dp.sl, dev, n, c->stream);
+    int le = exchange_state(c, dev, true);
     if (le) e = (cudaError_t)le;
     if (e == cudaSuccess && !on_device)
       e = cudaMemcpyAsync(dst, dev, fdlb_state_bytes(c), cudaMemcpyDeviceToHost, c->stream);
@@ -755,15 +778,14 @@ int fdlb_set_state(fdlb_ctx* c, const void* src, int on_device) {
   cudaError_t e = cudaSuccess;
   if (c->precision == FDLB_MIXED) {
     // each binary64 value v becomes hi = v rounded, lo = (v - hi) rounded
-    const double* dev = (const double*)src;
+    double* dev = (double*)src;  // (read only)
     if (!on_device) {
       e = cudaMemcpyAsync(mixed_exchange_buffer(c), src, fdlb_state_bytes(c),
                           cudaMemcpyHostToDevice, c->stream);
       dev = mixed_exchange_buffer(c);
     }
-    const int64_t n = (int64_t)c->dp.P * c->dp.N;
     if (e == cudaSuccess) {
-      int le = fdlb::launch_double_to_pair(dev, c->dp.sh, c->dp.sl, n, c->stream);
+      int le = exchange_state(c, dev, false);
       if (le) e = (cudaError_t)le;
     }
   } else {
@@ -884,7 +906,8 @@ int fdlb_create_batch(int nprob, const int64_t* nx, const double* gamma, double 
   }
   p.bgrid = 4 * c->nsm;
   const size_t pstat_bytes = ((size_t)nprob * sizeof(unsigned) + 255) / 256 * 256;
-  const Layout lay = buffer_layout(precision, p.P, total);
+  set_strides(p);
+  const Layout lay = buffer_layout(precision, p.P, total, p.NS);
   c->buf_bytes = lay.total + pstat_bytes;
   e = cudaMalloc(&c->buf, c->buf_bytes);
   if (e == cudaSuccess) e = cudaMalloc(&c->probs_dev, nprob * sizeof(fdlb::BatchProblem));
@@ -966,13 +989,7 @@ int fdlb_autotune(fdlb_ctx* c, int trial_steps, int* variant_out, int* ctas_per_
   cudaError_t e = cudaMalloc(&saved, bytes);
   if (e != cudaSuccess) return set_err(c, FDLB_ENOMEM, "autotune buffer: %s", cudaGetErrorString(e));
   auto put_state = [&](bool restore) -> cudaError_t {
-    if (c->precision == FDLB_MIXED) {
-      const int64_t n = (int64_t)c->dp.P * c->dp.N;
-      return (cudaError_t)(restore ? fdlb::launch_double_to_pair((const double*)saved, c->dp.sh,
-                                                                 c->dp.sl, n, c->stream)
-                                   : fdlb::launch_pair_to_double(c->dp.sh, c->dp.sl,
-                                                                 (double*)saved, n, c->stream));
-    }
+    if (c->precision == FDLB_MIXED) return (cudaError_t)exchange_state(c, (double*)saved, !restore);
     return restore ? cudaMemcpyAsync(c->dp.F, saved, bytes, cudaMemcpyDeviceToDevice, c->stream)
                    : cudaMemcpyAsync(saved, c->dp.F, bytes, cudaMemcpyDeviceToDevice, c->stream);
   };

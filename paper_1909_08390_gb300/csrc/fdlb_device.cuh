@@ -80,6 +80,13 @@ struct Geo {
   int prob;  // batch problem index, -1 for a single-problem context
 };
 
+// Where cell c of the grid sits in a population of a FDLB_MIXED context.
+__device__ __forceinline__ int64_t mixed_cell(const DevParams& p, int64_t c) {
+  if (p.pitch == p.nx) return c;
+  const int64_t y = c / p.nx;
+  return y * p.pitch + (c - y * p.nx);
+}
+
 // One axis of the Hermite-expanded equilibrium (Eq. gExpanded):
 // g_k = sum_{l<Q} [w_k He_l(p_k)/l!] a_l(u, T) with
 // a_l = sum_s l!/(2^s s!(l-2s)!) (T-1)^s u^(l-2s), generated by the

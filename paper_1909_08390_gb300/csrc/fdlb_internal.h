@@ -105,8 +105,15 @@ struct DevParams {
   // relative to the state's sh: R3 = sh + r3l, A4' = sh + a4l (then
   // R4 = sh + a4l), A_fin = sh + afl; dm holds D = R - F_eq of the last
   // stage; fa, fb, fc the low parts F2 - sh, F3 - sh, F4 - sh that stages 3,
-  // 4 and final advect.  mhi[4][N] holds per cell the binary64 moment sums
+  // 4 and final advect.  mhi[4][NS] holds per cell the binary64 moment sums
   // (n, jx, jy, e) of sh.
+  // 2-D arrays have rows of `pitch` cells and populations of NS cells; where
+  // `padded` both sides are rounded up to whole 16-cell tiles, so that every
+  // copy and store of a tile is whole and 16-byte aligned (the cells past nx
+  // and ny hold nothing and feed nothing).  1-D: pitch = nx, NS = N.
+  int pitch, padded;
+  int64_t NS;
+  double* xstate;  // binary64 populations F[P][N] (kStateOut, kStateIn)
   float *sh, *sl, *nh, *nl;
   float *r3l, *a4l, *afl;
   float *dm, *fa, *fb, *fc;
@@ -118,7 +125,9 @@ struct DevParams {
 constexpr int kBatchVariants = 3;
 int batch_tile_cells(int variant);
 
-enum Stage { kPrep = 0, kStage3 = 1, kStage4 = 2, kFinal = 3 };
+// kStateOut, kStateIn: the binary32-pair state of a FDLB_MIXED context to and
+// from the binary64 array xstate.
+enum Stage { kPrep = 0, kStage3 = 1, kStage4 = 2, kFinal = 3, kStateOut = 4, kStateIn = 5 };
 
 // Kernel launchers (fdlb_kernels.cu).  Each returns a cudaError_t value.
 bool supported_lattice(int d, int Qp, int Qc);
@@ -139,8 +148,6 @@ int launch_batch_init(const DevParams& p, cudaStream_t s);
 int mixed_setup(const DevParams& p);
 int launch_mixed_stage(const DevParams& p, int stage, cudaStream_t s);
 int launch_mixed_batch_stage(const DevParams& p, int stage, cudaStream_t s);
-// the binary32-pair state of FDLB_MIXED contexts <-> binary64 values
-int launch_pair_to_double(const float* hi, const float* lo, double* out, int64_t n, cudaStream_t s);
-int launch_double_to_pair(const double* in, float* hi, float* lo, int64_t n, cudaStream_t s);
+int launch_mixed_exchange(const DevParams& p, bool out, cudaStream_t s);
 
 }  // namespace fdlb

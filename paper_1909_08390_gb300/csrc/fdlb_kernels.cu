@@ -694,6 +694,7 @@ template <typename S, int DIM, int QP, int QC>
 __device__ __forceinline__ void store_state(const DevParams& p,
                                             const EqCellS<DIM, QP, QC, double>& eq, int64_t c) {
   using L = Lat<DIM, QP, QC>;
+  const int64_t m = sizeof(S) == 8 ? c : mixed_cell(p, c);
 #pragma unroll
   for (int pop = 0; pop < L::P; ++pop) {
     const double v = feq_of<DIM, QP, QC, double>(eq, pop);
@@ -701,8 +702,8 @@ __device__ __forceinline__ void store_state(const DevParams& p,
       ((double*)p.F)[pop * p.N + c] = v;
     } else {
       const float h = (float)v;
-      p.sh[pop * p.N + c] = h;
-      p.sl[pop * p.N + c] = (float)(v - (double)h);
+      p.sh[pop * p.NS + m] = h;
+      p.sl[pop * p.NS + m] = (float)(v - (double)h);
     }
   }
 }
@@ -795,8 +796,9 @@ __global__ void mixed_moments_kernel(const __grid_constant__ DevParams p, double
   using L = Lat<DIM, QP, QC>;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= p.N) return;
-  Moments m = {p.mhi[c], p.mhi[p.N + c], p.mhi[2 * p.N + c], p.mhi[3 * p.N + c]};
-  for (int pop = 0; pop < L::P; ++pop) accumulate<DIM, QP, QC>(p, m, pop, (double)p.sl[pop * p.N + c]);
+  const int64_t i = mixed_cell(p, c);
+  Moments m = {p.mhi[i], p.mhi[p.NS + i], p.mhi[2 * p.NS + i], p.mhi[3 * p.NS + i]};
+  for (int pop = 0; pop < L::P; ++pop) accumulate<DIM, QP, QC>(p, m, pop, (double)p.sl[pop * p.NS + i]);
   double nn, vx, vy, TT;
   const double invDK = p.nprob > 0 ? p.probs[find_problem(p, c)].invDK : p.invDK;
   moments_to_nut<DIM>(invDK, m, nn, vx, vy, TT);
@@ -1014,6 +1016,7 @@ bool supported_lattice(int d, int Qp, int Qc) {
 }
 
 int launch_stage(const DevParams& p, int stage, cudaStream_t s) {
+  if (stage == kStateOut || stage == kStateIn) return launch_mixed_exchange(p, stage == kStateOut, s);
 #define X(D_, P_, C_) \
   if (p.d == D_ && p.Qp == P_ && p.Qc == C_) return launch_stage_t<D_, P_, C_>(p, stage, s);
   FDLB_LATTICES(X)

@@ -35,9 +35,13 @@
 // copies (chunks of 4 cells, fdlb_tile.cuh), and pass 2 of a tile inside
 // the grid streams its values through the then idle staging buffers, a ring
 // of four chunks copied three steps ahead; elsewhere copies are per cell.
-// Grids whose sides are multiples of the 16-cell tile, on lattices whose
-// populations fill whole groups, run an instance compiled without the
-// per-cell paths (FAST): unexecuted code in these kernels costs time.
+// Lattices whose populations fill whole groups run an instance compiled
+// without the per-cell paths (FAST): unexecuted code in these kernels costs
+// time.  The arrays of a 2-D grid are padded to whole 16-cell tiles (DevParams
+// ::padded), so that every tile's chunks are whole and aligned; only periodic
+// grids whose rows hold no multiple of 4 cells, and grids too thin to pad,
+// still copy cell by cell.  333 x 517 cells, 128 populations: 0.82 ms a step
+// padded, 1.86 cell by cell.
 //
 // Moments: R3's and R4's are the binary64 per-cell sums of sh (mhi, left by
 // the previous final stage) plus binary32 sums of their low parts; the final
@@ -268,7 +272,7 @@ __device__ __forceinline__ void relax_cell(const DevParams& p, double kchi, doub
   }
   EqFac<DIM, QP, QC> fac;
   eq_factors<DIM, QP, QC>(p, kchi, n, ux, uy, T, fac);
-  const int64_t N = p.N;
+  const int64_t N = p.NS;
   using RW = EqRows<DIM, QP, QC>;
   // row by row, the next row's values loaded before this row is computed
   float ca[kMaxRow], cb[kMaxRow], na[kMaxRow], nb[kMaxRow];
@@ -321,7 +325,7 @@ __device__ __forceinline__ DF pick_df(const DF (&a)[Q], int k) {
 
 template <int DIM, int QP, int QC, int TX, int TY, int NT>
 __device__ __forceinline__ void relax_tile_streamed(const DevParams& p, double kchi, double invDK,
-                                                    int prob, const double (&mom)[2][4],
+                                                    const bool (&valid)[2], const double (&mom)[2][4],
                                                     int64_t N, int64_t cell0, int nx,
                                                     const float* __restrict__ ain,
                                                     const float* __restrict__ bin, float kd,
@@ -370,10 +374,7 @@ __device__ __forceinline__ void relax_tile_streamed(const DevParams& p, double k
       const double uy = DIM == 2 ? jy * inv_n : 0.0;
       const double T = (e - fma(jx, ux, jy * uy)) * inv_n * invDK;
       const bool ok = n > 0.0 && T > 0.0 && isfinite(n) && isfinite(T) && isfinite(ux) && isfinite(uy);
-      if (!ok) {
-        atomicOr(p.status, 1u);
-        if (prob >= 0) atomicOr(&p.pstatus[prob], 1u);
-      }
+      if (!ok && (k == 0 ? valid[0] : valid[1])) atomicOr(p.status, 1u);
       eq_factors<DIM, QP, QC>(p, kchi, n, ux, uy, T, fac);
       const int ci = k * HALF + tid;
       mycell = cell0 + (int64_t)(ci / TX) * nx + ci % TX;
@@ -473,9 +474,8 @@ struct MixSmem {
 
 // One tile of one stage.  Ends with every thread past its last use of the
 // shared memory, so a persistent CTA may start its next tile at once.
-// FAST: a 2-D grid whose sides are multiples of the tile's and whose
-// populations fill whole groups (every tile full, every row 16-byte
-// aligned), compiled without the per-cell copy and relaxation paths (the
+// FAST: a 2-D grid padded to whole tiles whose populations fill whole groups
+// (every chunk whole and 16-byte aligned), compiled without the per-cell copy and relaxation paths (the
 // kernels are sensitive to code size).
 template <int DIM, int QP, int QC, int STAGE, int VAR, bool FAST = false>
 __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, int x0, int y0,
@@ -499,14 +499,16 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
   // (final stage), left by the previous kernel's pass 2
   const float* __restrict__ const fin = STAGE == kStage3 ? p.fa : (STAGE == kStage4 ? p.fb : p.fc);
   const int tid = threadIdx.x;
-  const int64_t N = p.N;
+  const int64_t N = p.NS;
+  const int pitch = DIM == 2 ? p.pitch : geo.nx;  // row pitch
 
   // chunked landing (16-byte copies) for 2-D grids whose rows, and so all
-  // chunk addresses, are 16-byte aligned; else cell by cell
+  // chunk addresses, are 16-byte aligned (periodic ones wrap whole chunks);
+  // else cell by cell
   constexpr bool kCh = M::NCL > 0;
   constexpr bool kFast = FAST && DIM == 2 && kCh && L::P % G == 0;
   static_assert(!FAST || kFast, "FAST needs 2-D chunked tiles and whole groups");
-  const bool chunked = kFast || (kCh && (geo.nx % 4) == 0 && (geo.base % 4) == 0);
+  const bool chunked = kFast || (kCh && pitch % 4 == 0 && (p.bc != 1 || geo.nx % 4 == 0));
   // this thread's staged cells: tile offset and landing slot (-1: none);
   // cell by cell, slot e holds staged cell e, and 1-D keeps its offset from
   // geo.base (2-D grids landed cell by cell recompute it)
@@ -532,7 +534,7 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
 #pragma unroll
     for (int i = 0; i < 2; ++i)
       if (chunked && tid + i * NT < NCHK)
-        go[i] = chunk_offset(tid + i * NT, TX, TY, x0, y0, geo.nx, geo.ny, p.bc);
+        go[i] = chunk_offset(tid + i * NT, TX, TY, x0, y0, geo.nx, geo.ny, p.bc, pitch);
   }
   // own cells of this thread: tid + k NT (coalesced in both passes); a slot
   // past the tile's cells takes cell 0's indices (its lane computes on them
@@ -547,7 +549,7 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
     lxs[k] = c % TX;
     lys[k] = c / TX;
     valid[k] = (ci < CELLS) && (x0 + lxs[k] < geo.nx) && (y0 + lys[k] < geo.ny);
-    cell[k] = geo.base + (int64_t)(y0 + lys[k]) * geo.nx + (x0 + lxs[k]);
+    cell[k] = geo.base + (int64_t)(y0 + lys[k]) * pitch + (x0 + lxs[k]);
   }
   // moment sums: stages 3 and 4 sum the low parts of R3, R4 plainly; the
   // final stage sums the new sh error-free (mom) and the new sl plainly
@@ -585,7 +587,7 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
   // first cell.  1-D tiles take none, so that a 1-D problem gives the same
   // bits whatever its tiling (batches and single problems use different
   // tile lengths).
-  const int64_t cref = geo.base + (int64_t)y0 * geo.nx + x0;
+  const int64_t cref = geo.base + (int64_t)y0 * pitch + x0;
 
   const int tg = tid / (NLINE * NSEG);  // the thread's population in a group (march)
   const int tline = (tid / NSEG) % NLINE;
@@ -617,7 +619,7 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
             } else {
               int r, c;
               staged_pos(tid + j * NT, DIM, TX, TY, r, c);
-              o = wrap_or_clamp(y0 - H + r, geo.ny, p.bc) * geo.nx +
+              o = wrap_or_clamp(y0 - H + r, geo.ny, p.bc) * pitch +
                   wrap_or_clamp(x0 - H + c, geo.nx, p.bc);
             }
             cp_async(&sm.rawh[g][loff[j]], srch + o);
@@ -635,8 +637,8 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
   // A 2-D tile wholly inside a grid of 16-byte aligned rows copies them as
   // 16-byte chunks of 4 cells, any thread any chunk (the barrier before
   // pass 1 orders them).
-  const bool own16 = kFast || (DIM == 2 && TX % 4 == 0 && (geo.nx % 4) == 0 && (geo.base % 4) == 0 &&
-                     x0 + TX <= geo.nx && y0 + TY <= geo.ny);
+  const bool own16 = kFast || (DIM == 2 && TX % 4 == 0 &&
+                               (p.padded || (pitch % 4 == 0 && x0 + TX <= geo.nx && y0 + TY <= geo.ny)));
   auto prefetch_own = [&](int gfirst) {
     const float* const src[3] = {p.dm, STAGE == kStage3 ? p.sl : (STAGE == kStage4 ? p.a4l : p.afl),
                                  STAGE == kStage4 ? p.afl : Sh};
@@ -652,7 +654,7 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
           const int row = cq / (TX / 4), c4 = (cq % (TX / 4)) * 4;
           const float* sa = a == 0 ? src[0] : (a == 1 ? src[1] : src[M::NOWN - 1]);
           cp_async16(&sm.own[a][g][row * TX + c4],
-                     sa + (int64_t)(gfirst + g) * N + geo.base + (int64_t)(y0 + row) * geo.nx + x0 + c4);
+                     sa + (int64_t)(gfirst + g) * N + geo.base + (int64_t)(y0 + row) * pitch + x0 + c4);
         }
         cp_async_commit();
         return;
@@ -867,8 +869,8 @@ __device__ __forceinline__ void mixed_tile(const DevParams& p, const Geo& geo, i
       // free once pass 1 has passed its last barrier
       static_assert(sizeof(float) * 4 * 2 * kMaxRow * NT <= offsetof(M, coef),
                     "the ring fits in the staging buffers");
-      relax_tile_streamed<DIM, QP, QC, TX, TY, NT>(p, geo.kchi, geo.invDK, geo.prob, mm, N,
-                                                   geo.base + (int64_t)y0 * geo.nx + x0, geo.nx,
+      relax_tile_streamed<DIM, QP, QC, TX, TY, NT>(p, geo.kchi, geo.invDK, valid, mm, N,
+                                                   geo.base + (int64_t)y0 * pitch + x0, pitch,
                                                    ain, bin, kd, fout, &sm.rawh[0][0]);
       return;
     }
@@ -946,26 +948,27 @@ __device__ __forceinline__ int problem_of(const DevParams& p, int64_t c) {
 template <int DIM, int QP, int QC>
 __global__ void mixed_prep_kernel(const __grid_constant__ DevParams p) {
   using L = Lat<DIM, QP, QC>;
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= p.N) return;
+  const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (cell >= p.N) return;
+  const int64_t c = mixed_cell(p, cell);
   MomentsF m = {};
   MomL lm = {};
   for (int pop = 0; pop < L::P; ++pop) {
-    accumulate<DIM, QP, QC>(p, m, pop, p.sh[pop * p.N + c]);
-    accum_low<DIM, QP, QC>(p, lm, pop, p.sl[pop * p.N + c]);
+    accumulate<DIM, QP, QC>(p, m, pop, p.sh[pop * p.NS + c]);
+    accum_low<DIM, QP, QC>(p, lm, pop, p.sl[pop * p.NS + c]);
   }
   Geo geo{p.nx, p.ny, 0, p.kchi, p.invDK, p.dtdx, p.dtdy, -1};
   if (p.nprob > 0) {
-    const int b = problem_of(p, c);
+    const int b = problem_of(p, cell);
     geo.kchi = p.probs[b].kchi;
     geo.invDK = p.probs[b].invDK;
     geo.prob = b;
   }
   const Moments mh = to_fp64(m);
   p.mhi[c] = mh.n;
-  p.mhi[p.N + c] = mh.jx;
-  p.mhi[2 * p.N + c] = mh.jy;
-  p.mhi[3 * p.N + c] = mh.e;
+  p.mhi[p.NS + c] = mh.jx;
+  p.mhi[2 * p.NS + c] = mh.jy;
+  p.mhi[3 * p.NS + c] = mh.e;
   relax_cell<DIM, QP, QC>(p, geo.kchi, geo.invDK, geo.prob, mh.n + (double)lm.n,
                           mh.jx + (double)lm.jx, mh.jy + (double)lm.jy, mh.e + (double)lm.e, p.sh,
                           p.sl, (float)(1.0 - p.sc.c2), p.fa, c);
@@ -1067,8 +1070,9 @@ int launch_t(const DevParams& p, int stage, cudaStream_t s) {
     }
   }
   if constexpr (fast_lattice<DIM, QP, QC>()) {
-    // every tile full: the instance without the per-cell paths
-    if (p.nx % TileCfg<2, 0>::TX == 0 && p.ny % TileCfg<2, 0>::TY == 0)
+    // whole tiles in memory and whole chunks at the edges: the instance
+    // without the per-cell paths
+    if (p.padded && (p.bc != 1 || p.nx % 4 == 0))
       return launch_tv<DIM, QP, QC, 0, true>(p, stage, s);
   }
   return launch_tv<DIM, QP, QC, 0>(p, stage, s);
@@ -1107,18 +1111,24 @@ int launch_batch_t(const DevParams& p, int stage, cudaStream_t s) {
 
 // ---- the state as binary64 values (fdlb_get_state / fdlb_set_state) ------
 
-__global__ void pair_to_double_kernel(const float* __restrict__ hi, const float* __restrict__ lo,
-                                      double* __restrict__ out, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (double)hi[i] + (double)lo[i];  // the pair's exact sum, rounded once
+// population blockIdx.y, cells along x
+__global__ void state_out_kernel(const __grid_constant__ DevParams p) {
+  const float* __restrict__ const hi = p.sh + blockIdx.y * p.NS;
+  const float* __restrict__ const lo = p.sl + blockIdx.y * p.NS;
+  double* __restrict__ const out = p.xstate + blockIdx.y * p.N;
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = mixed_cell(p, c);
+    out[c] = (double)hi[i] + (double)lo[i];  // the pair's exact sum, rounded once
+  }
 }
 
-__global__ void double_to_pair_kernel(const double* __restrict__ in, float* __restrict__ hi,
-                                      float* __restrict__ lo, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double v = in[i];
+__global__ void state_in_kernel(const __grid_constant__ DevParams p) {
+  float* __restrict__ const hi = p.sh + blockIdx.y * p.NS;
+  float* __restrict__ const lo = p.sl + blockIdx.y * p.NS;
+  const double* __restrict__ const in = p.xstate + blockIdx.y * p.N;
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = mixed_cell(p, c);
+    const double v = in[c];
     const float h = (float)v;
     hi[i] = h;
     lo[i] = (float)(v - (double)h);
@@ -1163,14 +1173,11 @@ int launch_mixed_batch_stage(const DevParams& p, int stage, cudaStream_t s) {
   return (int)cudaErrorInvalidValue;
 }
 
-int launch_pair_to_double(const float* hi, const float* lo, double* out, int64_t n,
-                          cudaStream_t s) {
-  pair_to_double_kernel<<<1024, 256, 0, s>>>(hi, lo, out, n);
-  return (int)cudaGetLastError();
-}
-
-int launch_double_to_pair(const double* in, float* hi, float* lo, int64_t n, cudaStream_t s) {
-  double_to_pair_kernel<<<1024, 256, 0, s>>>(in, hi, lo, n);
+int launch_mixed_exchange(const DevParams& p, bool out, cudaStream_t s) {
+  const int64_t nb = (p.N + 255) / 256;
+  const dim3 grid((unsigned)(nb < 1024 ? nb : 1024), p.P);
+  if (out) state_out_kernel<<<grid, 256, 0, s>>>(p);
+  else state_in_kernel<<<grid, 256, 0, s>>>(p);
   return (int)cudaGetLastError();
 }
 

@@ -58,14 +58,17 @@ FDLB_HD void staged_pos(int e, int dim, int TX, int TY, int& r, int& c) {
 // then the tile's TY rows from column x0 - 8 to x0 + TX + 8 ((TX+16)/4
 // chunks, the 5-cell halos rounded out to whole chunks), then the kGhost rows
 // below.  chunk_offset gives chunk q's first cell as an offset from the
-// population's first cell: rows clamp (outlet) or wrap (periodic) as a
-// whole; periodic columns wrap chunk by chunk; an outlet chunk reaching past
-// the left or right edge is not copied (-1), and chunk_slot sends the cells
+// population's first cell (rows of `pitch` cells, a multiple of 4; 0: nx):
+// rows clamp (outlet) or wrap (periodic) as a whole; periodic columns wrap
+// chunk by chunk (nx a multiple of 4); an outlet chunk past the left or right
+// edge is not copied (-1; one that holds the edge column is, with the row's
+// padding), and chunk_slot sends the cells
 // that would read it to the edge column instead (the ghost value), which the
 // row's other chunks hold.  chunk_slot gives the landing slot of staged
 // position (r, c) (the tile's first cell at (kGhost, kGhost)).
 FDLB_HD int chunk_count(int TX, int TY) { return (2 * kGhost * TX + TY * (TX + 16)) / 4; }
-FDLB_HD int chunk_offset(int q, int TX, int TY, int x0, int y0, int nx, int ny, int bc) {
+FDLB_HD int chunk_offset(int q, int TX, int TY, int x0, int y0, int nx, int ny, int bc,
+                         int pitch = 0) {
   const int top = kGhost * TX / 4, mid = TY * (TX + 16) / 4;
   int r, col;
   if (q < top) {
@@ -79,8 +82,9 @@ FDLB_HD int chunk_offset(int q, int TX, int TY, int x0, int y0, int nx, int ny, 
     col = x0 + ((q - top - mid) % (TX / 4)) * 4;
   }
   const int rr = wrap_or_clamp(y0 - kGhost + r, ny, bc);
-  if (bc == 1) return rr * nx + wrap_or_clamp(col, nx, 1);
-  return (col >= 0 && col + 4 <= nx) ? rr * nx + col : -1;
+  if (pitch == 0) pitch = nx;
+  if (bc == 1) return rr * pitch + wrap_or_clamp(col, nx, 1);
+  return (col >= 0 && col < nx && col + 4 <= pitch) ? rr * pitch + col : -1;
 }
 FDLB_HD int chunk_slot(int r, int c, int TX, int TY, int x0, int nx, int bc) {
   int cc = x0 - kGhost + c;

@@ -81,8 +81,8 @@ TRAFFIC_BYTES = {
 
 
 # The sources the stage kernels are compiled from.
-STAGE_KERNEL_SOURCES = ("fdlb_device.cuh", "fdlb_internal.h", "fdlb_kernels.cu", "fdlb_mixed.cu",
-                        "fdlb_mp9.cuh", "fdlb_mp9i.cuh", "fdlb_tile.cuh")
+STAGE_KERNEL_SOURCES = ("fdlb_cvt.cuh", "fdlb_device.cuh", "fdlb_internal.h", "fdlb_kernels.cu",
+                        "fdlb_mixed.cu", "fdlb_mp9.cuh", "fdlb_mp9i.cuh", "fdlb_tile.cuh")
 
 
 def _kernel_sources_sha256(root=None):

@@ -24,7 +24,7 @@ SOURCES = ["fdlb_kernels.cu", "fdlb_mixed.cu", "fdlb_api.cpp", "fdlb_noalloc.cu"
            "fdlb_peak.cu"]
 HEADERS = [os.path.join(CSRC, "fdlb_internal.h"), os.path.join(CSRC, "fdlb_ctx.h"),
            os.path.join(CSRC, "fdlb_device.cuh"),
-           os.path.join(CSRC, "fdlb_mp9.cuh"), os.path.join(CSRC, "fdlb_mp9i.cuh"),
+           os.path.join(CSRC, "fdlb_mp9.cuh"), os.path.join(CSRC, "fdlb_mp9i.cuh"), os.path.join(CSRC, "fdlb_cvt.cuh"),
            os.path.join(CSRC, "fdlb_tile.cuh"),
            os.path.join(INCLUDE, "fdlb.h")]
 

@@ -9,6 +9,7 @@
 
 #include <cstdint>
 
+#include "fdlb_cvt.cuh"
 #include "fdlb_internal.h"
 #include "fdlb_mp9.cuh"
 #include "fdlb_tile.cuh"

@@ -701,9 +701,7 @@ __device__ __forceinline__ void store_state(const DevParams& p,
     if constexpr (sizeof(S) == 8) {
       ((double*)p.F)[pop * p.N + c] = v;
     } else {
-      const float h = (float)v;
-      p.sh[pop * p.NS + m] = h;
-      p.sl[pop * p.NS + m] = (float)(v - (double)h);
+      split_pair(v, p.sh[pop * p.NS + m], p.sl[pop * p.NS + m]);
     }
   }
 }
@@ -761,6 +759,15 @@ struct RiemannArgs {
   double sx, sy;  // membranes in cell units (split_in_cells)
 };
 
+// index of the state that cell (x, y) takes
+template <int DIM>
+__device__ __forceinline__ int riemann_side(const RiemannArgs& a, int x, int y) {
+  const bool right = (double)x + 0.5 >= a.sx;
+  if (DIM == 1) return right ? 1 : 0;
+  const bool upper = (double)y + 0.5 >= a.sy;
+  return upper ? (right ? 0 : 1) : (right ? 3 : 2);
+}
+
 template <int DIM, int QP, int QC, typename S>
 __global__ void init_riemann_kernel(const __grid_constant__ DevParams p,
                                     const __grid_constant__ RiemannArgs a) {
@@ -768,14 +775,7 @@ __global__ void init_riemann_kernel(const __grid_constant__ DevParams p,
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= p.N) return;
   const int x = (int)(c % p.nx), y = (int)(c / p.nx);
-  const bool right = (double)x + 0.5 >= a.sx;
-  int q;
-  if (DIM == 1) {
-    q = right ? 1 : 0;
-  } else {
-    const bool upper = (double)y + 0.5 >= a.sy;
-    q = upper ? (right ? 0 : 1) : (right ? 3 : 2);
-  }
+  const int q = riemann_side<DIM>(a, x, y);
   const double rho = a.st[q][0];
   const double ux = a.st[q][1];
   const double uy = DIM == 2 ? a.st[q][2] : 0.0;
@@ -785,6 +785,47 @@ __global__ void init_riemann_kernel(const __grid_constant__ DevParams p,
   EqCellS<DIM, QP, QC, double> eq;  // binary64 products, rounded once on store
   to_storage(eq64, eq);
   store_state<S>(p, eq, c);
+}
+
+// The same on large grids: the data hold 2 or 4 states, so each CTA forms their
+// populations once and its threads copy them (a state's populations took one
+// thread 250 to 800 binary64 operations for every cell: 5.3 of the 11.6 ms of
+// setting 2048 x 2048 x 128 mixed populations).
+template <int DIM, int QP, int QC, typename S>
+__global__ void __launch_bounds__(256) fill_riemann_kernel(const __grid_constant__ DevParams p,
+                                                           const __grid_constant__ RiemannArgs a) {
+  using L = Lat<DIM, QP, QC>;
+  __shared__ double val[sizeof(S) == 8 ? 4 : 1][L::P];
+  __shared__ float2 pair[sizeof(S) == 8 ? 1 : 4][L::P];
+  if (threadIdx.x < a.nq) {
+    const int q = threadIdx.x;
+    const double rho = a.st[q][0], P = a.st[q][DIM == 2 ? 3 : 2];
+    EqCell<DIM, QP, QC> eq64;
+    make_eq_nut<DIM, QP, QC>(p, p.kchi, rho, a.st[q][1], DIM == 2 ? a.st[q][2] : 0.0, P / rho, eq64);
+    EqCellS<DIM, QP, QC, double> eq;
+    to_storage(eq64, eq);
+#pragma unroll
+    for (int pop = 0; pop < L::P; ++pop) {
+      const double v = feq_of<DIM, QP, QC, double>(eq, pop);
+      if constexpr (sizeof(S) == 8) val[q][pop] = v;
+      else split_pair(v, pair[q][pop].x, pair[q][pop].y);
+    }
+  }
+  __syncthreads();
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += (int64_t)gridDim.x * blockDim.x) {
+    const int x = (int)(c % p.nx), y = (int)(c / p.nx);
+    const int q = riemann_side<DIM>(a, x, y);
+    const int64_t m = sizeof(S) == 8 ? c : mixed_cell(p, c);
+#pragma unroll 8
+    for (int pop = 0; pop < L::P; ++pop) {
+      if constexpr (sizeof(S) == 8) {
+        ((double*)p.F)[pop * p.N + m] = val[q][pop];
+      } else {
+        p.sh[pop * p.NS + m] = pair[q][pop].x;
+        p.sl[pop * p.NS + m] = pair[q][pop].y;
+      }
+    }
+  }
 }
 
 // Moments of a binary32-pair state: the binary64 sums of the high parts
@@ -798,7 +839,24 @@ __global__ void mixed_moments_kernel(const __grid_constant__ DevParams p, double
   if (c >= p.N) return;
   const int64_t i = mixed_cell(p, c);
   Moments m = {p.mhi[i], p.mhi[p.NS + i], p.mhi[2 * p.NS + i], p.mhi[3 * p.NS + i]};
-  for (int pop = 0; pop < L::P; ++pop) accumulate<DIM, QP, QC>(p, m, pop, (double)p.sl[pop * p.NS + i]);
+  if constexpr (DIM == 2 && QP == 8) {
+    // row and column sums (GroupMoments): 1.6 binary64 operations a population
+    using GM = GroupMoments<QP, QC>;
+    GM g = {};
+#pragma unroll 2
+    for (int gi = 0; gi < GM::NG; ++gi) {
+      const int g0 = GM::first(gi);
+      double v[kG];
+#pragma unroll
+      for (int j = 0; j < kG; ++j) v[j] = widen(p.sl[(g0 + j) * p.NS + i]);
+      g.add(p, g0, v);
+      g.fold(p, gi);
+    }
+    m = Moments{m.n + g.m.n, m.jx + g.m.jx, m.jy + g.m.jy, m.e + g.m.e};
+  } else {
+#pragma unroll 4
+    for (int pop = 0; pop < L::P; ++pop) accumulate<DIM, QP, QC>(p, m, pop, widen(p.sl[pop * p.NS + i]));
+  }
   double nn, vx, vy, TT;
   const double invDK = p.nprob > 0 ? p.probs[find_problem(p, c)].invDK : p.invDK;
   moments_to_nut<DIM>(invDK, m, nn, vx, vy, TT);
@@ -953,7 +1011,11 @@ template <int DIM, int QP, int QC>
 int launch_init_t(const DevParams& p, const RiemannArgs& a, cudaStream_t s) {
   const int nt = 128;
   const int64_t nb = (p.N + nt - 1) / nt;
-  if (p.precision == 1) init_riemann_kernel<DIM, QP, QC, float><<<(unsigned)nb, nt, 0, s>>>(p, a);
+  // from 2^16 cells on a CTA's own table (8 us) costs less than a cell's factors
+  if (p.N >= (1 << 16)) {
+    if (p.precision == 1) fill_riemann_kernel<DIM, QP, QC, float><<<608, 256, 0, s>>>(p, a);
+    else fill_riemann_kernel<DIM, QP, QC, double><<<608, 256, 0, s>>>(p, a);
+  } else if (p.precision == 1) init_riemann_kernel<DIM, QP, QC, float><<<(unsigned)nb, nt, 0, s>>>(p, a);
   else init_riemann_kernel<DIM, QP, QC, double><<<(unsigned)nb, nt, 0, s>>>(p, a);
   return (int)cudaGetLastError();
 }

@@ -953,6 +953,7 @@ __global__ void mixed_prep_kernel(const __grid_constant__ DevParams p) {
   const int64_t c = mixed_cell(p, cell);
   MomentsF m = {};
   MomL lm = {};
+#pragma unroll 8
   for (int pop = 0; pop < L::P; ++pop) {
     accumulate<DIM, QP, QC>(p, m, pop, p.sh[pop * p.NS + c]);
     accum_low<DIM, QP, QC>(p, lm, pop, p.sl[pop * p.NS + c]);
@@ -1111,14 +1112,16 @@ int launch_batch_t(const DevParams& p, int stage, cudaStream_t s) {
 
 // ---- the state as binary64 values (fdlb_get_state / fdlb_set_state) ------
 
-// population blockIdx.y, cells along x
+// population blockIdx.y, cells along x (several loads in flight a thread)
 __global__ void state_out_kernel(const __grid_constant__ DevParams p) {
   const float* __restrict__ const hi = p.sh + blockIdx.y * p.NS;
   const float* __restrict__ const lo = p.sl + blockIdx.y * p.NS;
   double* __restrict__ const out = p.xstate + blockIdx.y * p.N;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += step) {
     const int64_t i = mixed_cell(p, c);
-    out[c] = (double)hi[i] + (double)lo[i];  // the pair's exact sum, rounded once
+    out[c] = widen(hi[i]) + widen(lo[i]);  // the pair's exact sum, rounded once
   }
 }
 
@@ -1128,10 +1131,7 @@ __global__ void state_in_kernel(const __grid_constant__ DevParams p) {
   const double* __restrict__ const in = p.xstate + blockIdx.y * p.N;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = mixed_cell(p, c);
-    const double v = in[c];
-    const float h = (float)v;
-    hi[i] = h;
-    lo[i] = (float)(v - (double)h);
+    split_pair(in[c], hi[i], lo[i]);
   }
 }
 

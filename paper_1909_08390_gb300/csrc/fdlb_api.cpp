@@ -904,7 +904,10 @@ int fdlb_create_batch(int nprob, const int64_t* nx, const double* gamma, double 
     delete c;
     return cuda_err(nullptr, e, "device query");
   }
-  p.bgrid = 4 * c->nsm;
+  // a CTA per tile for most batches (a launch takes no more CTAs than tiles):
+  // 512 mixed problems 0.503 ms a step against 0.559 with 4 per SM, whose last
+  // round is partly empty and leaves 1 of the 5 CTAs an SM holds unused
+  p.bgrid = 64 * c->nsm;
   const size_t pstat_bytes = ((size_t)nprob * sizeof(unsigned) + 255) / 256 * 256;
   set_strides(p);
   const Layout lay = buffer_layout(precision, p.P, total, p.NS);

@@ -1033,7 +1033,7 @@ int launch_moments_t(const DevParams& p, double* n, double* ux, double* uy, doub
 template <int QP, int QC, int VAR>
 int launch_batch_stage_v(const DevParams& p, int stage, cudaStream_t s) {
   using C = Tile1<VAR>;
-  const int grid = p.bgrid > 0 ? p.bgrid : 1;
+  const int grid = p.bgrid < p.nwork ? p.bgrid : p.nwork;
   switch (stage) {
     case kPrep: return launch_prep<1, QP, QC>(p, s);
     case kStage3: batch_stage_kernel<QP, QC, kStage3, VAR><<<grid, C::NT, 0, s>>>(p); break;

@@ -1082,7 +1082,7 @@ int launch_t(const DevParams& p, int stage, cudaStream_t s) {
 template <int QP, int QC, int VAR>
 int launch_batch_v(const DevParams& p, int stage, cudaStream_t s) {
   using C = TileCfg<1, VAR>;
-  const int grid = p.bgrid > 0 ? p.bgrid : 1;
+  const int grid = p.bgrid < p.nwork ? p.bgrid : p.nwork;
   switch (stage) {
     case kPrep: return launch_prep<1, QP, QC>(p, s);
     case kStage3:

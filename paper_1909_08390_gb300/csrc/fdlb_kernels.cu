@@ -266,7 +266,7 @@ struct Smem2 {
 // during pass 2.
 // Measured at 512 x 512 x 128 populations, per step: 9.93 ms with the march in
 // binary64 (that pipe 78 % busy), 3.64 ms with every warp marching and
-// updating in turn (the pipes idle in turn), 3.29 ms so.  What bounds it now:
+// updating in turn (the pipes idle in turn), 3.16 ms so.  What bounds it now:
 // about 680 instructions per population-cell and stage at half the issue
 // rate, the integer pipe and the binary64 pipe each about half busy; 16 warps
 // a CTA wait on the fixed latency of 64-bit integer chains.
@@ -409,6 +409,18 @@ __global__ void __launch_bounds__(Tile2::NM + Tile2::NU, CTAS)
       for (int gi = 0; gi < GM::NG; ++gi, ++it) {
         const int b = it & 1, g0 = GM::first(gi);
         load(g0, in);
+        // the next group's inputs on their way to L2, a thread per tile row,
+        // population and array: the registers to load them ahead are not there
+        // (512 x 512: 3.28 -> 3.16 ms a step; grids of few tiles sit in L2)
+        if (CTAS == 2 && gi + 1 < GM::NG && tid < (STAGE == kStage4 ? 3 : 2) * 16 * kG) {
+          const int row = tid % 16, pop = GM::first(gi + 1) + tid / 16 % kG, arr = tid / (16 * kG);
+          const int xr = tile % ntx * TX, yr = tile / ntx * TY + row;
+          if (pop < L::P && yr < p.ny) {
+            const double* a = (const double*)(arr == 1 ? p.D : arr == 2 || STAGE == kFinal ? p.Af
+                                                          : STAGE == kStage3 ? p.F : p.A4);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(a + pop * N + (unsigned)(yr * p.nx + xr)));
+          }
+        }
         bar_sync(kFull + b, NM + NU);  // the group's flux differences are in
         double R[kG];
 #pragma unroll
@@ -946,7 +958,7 @@ int launch_stage_2d_c(const DevParams& p, int ntx, int ntiles, int nsm, cudaStre
 // Grids of no more tiles than SMs run one CTA per SM, whose threads then have
 // 128 registers; larger ones run two of 64 (some spills, twice the warps):
 // 96 x 70, 30 tiles, 0.165 against 0.178 ms a stage; 512 x 512, 1024 tiles,
-// 1.21 against 1.10.
+// 1.21 against 1.10 (before the inputs' prefetch).
 template <int QP, int QC, int STAGE>
 int launch_stage_2d(const DevParams& p, cudaStream_t s) {
   const int ntx = (p.nx + Tile2::TX - 1) / Tile2::TX, nty = (p.ny + Tile2::TY - 1) / Tile2::TY;

@@ -228,7 +228,8 @@ int fdlb_batch_offsets(const fdlb_ctx* ctx, int64_t* base);
 
 /* Autotuner of a batch context: times trial_steps steps of every tile shape
  * (cells per tile 127, 63, 255) and persistent-grid size (2, 4, 8, 16 CTAs
- * per SM) on the context's own problems, starting each trial from the
+ * per SM; 16 stands for a CTA per tile, 64 per SM at most, as a new context
+ * has it) on the context's own problems, starting each trial from the
  * current state, restores the state and keeps the fastest shape.  The
  * chosen shape is returned in *variant_out and *ctas_per_sm_out (either may
  * be NULL).  Allocates one temporary state copy. */

@@ -980,6 +980,10 @@ int fdlb_batch_offsets(const fdlb_ctx* c, int64_t* base) {
   return FDLB_OK;
 }
 
+// CTAs per SM that the autotuner's grid size k stands for: the largest is a
+// CTA per tile (64 per SM at most), as a context starts with.
+static int tuned_ctas(int k) { return k >= 16 ? 64 : k; }
+
 int fdlb_autotune(fdlb_ctx* c, int trial_steps, int* variant_out, int* ctas_per_sm_out) {
   if (!c) return set_err(nullptr, FDLB_EINVAL, "ctx is NULL");
   if (!c->batch) return set_err(c, FDLB_EINVAL, "autotuning applies to batch contexts");
@@ -1007,7 +1011,7 @@ int fdlb_autotune(fdlb_ctx* c, int trial_steps, int* variant_out, int* ctas_per_
     c->dp.variant = v;
     if ((rc = upload_work(c))) break;
     for (int k : ctas) {
-      c->dp.bgrid = k * c->nsm;
+      c->dp.bgrid = tuned_ctas(k) * c->nsm;
       e = put_state(true);
       int le = e == cudaSuccess ? launch_stage_any(c, fdlb::kPrep, c->stream) : 0;
       if (e == cudaSuccess) e = cudaEventRecord(t0, c->stream);
@@ -1029,7 +1033,7 @@ int fdlb_autotune(fdlb_ctx* c, int trial_steps, int* variant_out, int* ctas_per_
   // restore the state and adopt the fastest shape
   if (e == cudaSuccess && !rc) {
     c->dp.variant = best_v;
-    c->dp.bgrid = best_k * c->nsm;
+    c->dp.bgrid = tuned_ctas(best_k) * c->nsm;
     rc = upload_work(c);
     if (!rc) e = put_state(true);
   }

@@ -43,17 +43,15 @@ UNIT = "cell-velocity updates/s"
 # explicit parts taking the previous stage's D_i terms).  The limited MP
 # branch, divisions and per-cell equilibrium factors are not counted.
 FLOPS_PER_POP = {"stage3": 48 + 5 + 20, "stage4": 48 + 5 + 16, "final": 48 + 5 + 12}
-# The kernels are bound by GB300's binary64 pipe, which executes one add,
+# GB300's binary64 pipe executes one add,
 # multiply or fused multiply-add per lane slot (2 slots per SM and clock), so
-# the roofline counts binary64 operations, not flops.  Algorithmic operations
-# per population and launch: one MP-9 interface value per axis (x and y), 15
-# each (the new difference, the 8-term stencil, the curvature, the two DM
-# candidates, the MD and LC bounds, the clamped result); the flux difference 4
-# (two differences, a multiply, an fma); then the stage's explicit part,
-# moment sums and relaxation: stage 3 6 + 4 + 3, stage 4 4 + 4 + 3, final
-# 2 + 4 + 3.  The tiles' extra interface per line, the per-cell equilibrium
-# factors and divisions are not counted.
-FP64_OPS_PER_POP = {"stage3": 30 + 4 + 13, "stage4": 30 + 4 + 11, "final": 30 + 4 + 9}
+# the roofline counts binary64 operations, not flops.  The MP-9 march runs on
+# the integer pipes (64-bit fixed point); binary64 operations per population
+# and launch are the stage's explicit part, moment sums (1.6: row and column
+# sums of the 8 x 8 lattice) and relaxation: stage 3 6 + 1.6 + 2, stage 4
+# 4 + 1.6 + 2, final 2 + 1.6 + 2.  The per-cell equilibrium factors and
+# divisions (about 1.1 a population) are not counted.
+FP64_OPS_PER_POP = {"stage3": 9.6, "stage4": 7.6, "final": 5.6}
 # Algorithmic HBM bytes per population and launch (binary64): arrays read and
 # written once each by the kernel (stage 3: F2, F, D -> F3, A4, Af, D3;
 # stage 4: F3, A4, Af, D3 -> F4, Af, D4; final: F4, Af, D4 -> F, D, F2).
@@ -448,7 +446,7 @@ def run_ours(args, world, rank, local):
     dfma_rate, _ = fdlb.fdlb_measure_fp64_pipe(stream)
     meas_gops = dfma_rate / 1e9
     roofline = {
-        "bound": "alu", "kernel": f"stage_kernel<2,8,8,{names[top]}>",
+        "bound": "alu", "kernel": f"stage_kernel_2d<8,8,{names[top]}>",
         "achieved": achieved_gops, "peak": meas_gops, "unit": "G binary64 op/s",
         "frac": achieved_gops / meas_gops,
         "peak_source": "measured: fdlb_measure_fp64_pipe, 8 independent DFMA chains per thread, "

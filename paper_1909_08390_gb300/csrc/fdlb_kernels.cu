@@ -238,20 +238,25 @@ __device__ __forceinline__ void bar_arrive(int id, int n) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// Tile of 16 x 16 cells; 256 marching and 256 updating threads.
+// Tile of 16 x 16 cells (or 16 x 8, on small grids); a marching thread for
+// every 8-cell half line of a group's populations, an updating one for every
+// cell.
+template <int TY_>
 struct Tile2 {
-  static constexpr int TX = 16, TY = 16, NM = 256, NU = 256, SEG = 8;
+  static constexpr int TX = 16, TY = TY_, NM = 16 * TY, NU = 16 * TY, SEG = 8;
+  static_assert(TY == 8 || TY == 16, "lines of one or two halves");
   static constexpr int SX = TX + 2 * H + 1, SY = TY + 2 * H;  // padded row pitch
 };
-template <int QP, int QC>
+template <int QP, int QC, int TY>
 struct Smem2 {
+  using T2 = Tile2<TY>;
   static constexpr int P = Lat<2, QP, QC>::P;
-  int64_t tile[2][kG][Tile2::SY][Tile2::SX];  // cells + halo: binary64, then integers
+  int64_t tile[2][kG][T2::SY][T2::SX];  // cells + halo: binary64, then integers
   // flux differences along x and y, in units of the scale with exponent ex
   // (0: binary64 bits)
-  int64_t hx[2][kG][Tile2::TY][Tile2::TX + 1];
-  int64_t hy[2][kG][Tile2::TX][Tile2::TY + 1];
-  double fac[QP + (QC == QP ? 0 : QC)][Tile2::NU];
+  int64_t hx[2][kG][T2::TY][T2::TX + 1];
+  int64_t hy[2][kG][T2::TX][T2::TY + 1];
+  double fac[QP + (QC == QP ? 0 : QC)][T2::NU];
   AdvCoef coef[P];  // dt |p| / ds
   int cex[P];
   int ex[2][kG];
@@ -270,16 +275,16 @@ struct Smem2 {
 // about 680 instructions per population-cell and stage at half the issue
 // rate, the integer pipe and the binary64 pipe each about half busy; 16 warps
 // a CTA wait on the fixed latency of 64-bit integer chains.
-template <int QP, int QC, int STAGE, int CTAS>
-__global__ void __launch_bounds__(Tile2::NM + Tile2::NU, CTAS)
+template <int QP, int QC, int STAGE, int CTAS, int TY_>
+__global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
     stage_kernel_2d(const __grid_constant__ DevParams p, int ntx, int ntiles) {
   using L = Lat<2, QP, QC>;
   using GM = GroupMoments<QP, QC>;
-  using T2 = Tile2;
+  using T2 = Tile2<TY_>;
   constexpr int TX = T2::TX, TY = T2::TY, NM = T2::NM, NU = T2::NU;
   constexpr int kMarchBar = 1, kFull = 2, kEmpty = 4;  // + buffer
   extern __shared__ __align__(16) unsigned char smraw[];
-  auto& sm = *reinterpret_cast<Smem2<QP, QC>*>(smraw);
+  auto& sm = *reinterpret_cast<Smem2<QP, QC, TY_>*>(smraw);
   const int64_t N = p.N;
   const int items = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x * GM::NG;
   for (int pop = threadIdx.x; pop < L::P; pop += NM + NU)
@@ -292,11 +297,14 @@ __global__ void __launch_bounds__(Tile2::NM + Tile2::NU, CTAS)
     const int tid = threadIdx.x;
     const double* __restrict__ const adv =
         (const double*)(STAGE == kStage3 ? p.F2 : STAGE == kStage4 ? p.F3 : p.A4);
-    // the thread's half line: population tg of the group; one warp takes the
-    // x lines of a population, the next its y lines (16 lines a half-warp
-    // keep the 8-byte accesses free of bank conflicts)
-    const int tg = tid / 64, ln = tid % 16, s0 = (tid / 16 % 2) * T2::SEG;
-    const bool xline = (tid & 32) == 0;
+    // the thread's half line: population tg of the group; 16 x 16: one warp
+    // takes the x lines of a population, the next its y lines; 16 x 8: half a
+    // warp each (either way 16 lanes access 8-byte elements of distinct banks)
+    constexpr int PT = NM / kG;  // threads of a population
+    const int tg = tid / PT;
+    const bool xline = tid % PT < PT / 2;
+    const int ln = xline ? tid % TY : tid % TX;
+    const int s0 = (xline ? tid / TY % 2 : TY == 16 ? tid / 16 % 2 : 0) * T2::SEG;
     // the thread's staged cells (staged_pos skips the corners): ghosts by
     // index clamp or wrap
     constexpr int NST = TY * (TX + 2 * H) + 2 * H * TX;
@@ -380,7 +388,7 @@ __global__ void __launch_bounds__(Tile2::NM + Tile2::NU, CTAS)
       int64_t* out = xline ? &sm.hx[b][tg][ln][first] : &sm.hy[b][tg][ln][first];
       const int emax = sm.mx[b][tg] >> 20;
       const bool fixed = emax >= kQExpMin && emax <= kQExpMax;
-      if (tid % 64 == 0) sm.ex[b][tg] = fixed ? emax : 0;
+      if (tid % PT == 0) sm.ex[b][tg] = fixed ? emax : 0;
       if (pop < L::P) {
         if (fixed) mp9_march_delta_int<T2::SEG>(up, sgn * step, out, sgn);
         else mp9_march_delta_fp64((const double*)up, sgn * step, out, sgn, T2::SEG);
@@ -412,7 +420,7 @@ __global__ void __launch_bounds__(Tile2::NM + Tile2::NU, CTAS)
         // the next group's inputs on their way to L2, a thread per tile row,
         // population and array: the registers to load them ahead are not there
         // (512 x 512: 3.28 -> 3.16 ms a step; grids of few tiles sit in L2)
-        if (CTAS == 2 && gi + 1 < GM::NG && tid < (STAGE == kStage4 ? 3 : 2) * 16 * kG) {
+        if (CTAS == 2 && TY == 16 && gi + 1 < GM::NG && tid < (STAGE == kStage4 ? 3 : 2) * 16 * kG) {
           const int row = tid % 16, pop = GM::first(gi + 1) + tid / 16 % kG, arr = tid / (16 * kG);
           const int xr = tile % ntx * TX, yr = tile / ntx * TY + row;
           if (pop < L::P && yr < p.ny) {
@@ -944,31 +952,35 @@ int launch_prep(const DevParams& p, cudaStream_t s) {
   return (int)cudaGetLastError();
 }
 
-template <int QP, int QC, int STAGE, int CTAS>
-int launch_stage_2d_c(const DevParams& p, int ntx, int ntiles, int nsm, cudaStream_t s) {
-  constexpr int bytes = (int)sizeof(Smem2<QP, QC>);
-  const cudaError_t e = cudaFuncSetAttribute(stage_kernel_2d<QP, QC, STAGE, CTAS>,
+template <int QP, int QC, int STAGE, int CTAS, int TY>
+int launch_stage_2d_c(const DevParams& p, int ntx, int nsm, cudaStream_t s) {
+  using T2 = Tile2<TY>;
+  constexpr int bytes = (int)sizeof(Smem2<QP, QC, TY>);
+  const cudaError_t e = cudaFuncSetAttribute(stage_kernel_2d<QP, QC, STAGE, CTAS, TY>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return (int)e;
+  const int ntiles = ntx * ((p.ny + TY - 1) / TY);
   const int grid = ntiles < CTAS * nsm ? ntiles : CTAS * nsm;
-  stage_kernel_2d<QP, QC, STAGE, CTAS><<<grid, Tile2::NM + Tile2::NU, bytes, s>>>(p, ntx, ntiles);
+  stage_kernel_2d<QP, QC, STAGE, CTAS, TY><<<grid, T2::NM + T2::NU, bytes, s>>>(p, ntx, ntiles);
   return (int)cudaGetLastError();
 }
 
 // Grids of no more tiles than SMs run one CTA per SM, whose threads then have
-// 128 registers; larger ones run two of 64 (some spills, twice the warps):
-// 96 x 70, 30 tiles, 0.165 against 0.178 ms a stage; 512 x 512, 1024 tiles,
-// 1.21 against 1.10 (before the inputs' prefetch).
+// 128 registers, on tiles of 16 x 8 cells while these too have an SM each (a
+// stage's time is then one tile's); larger grids run two CTAs of 64 registers
+// (some spills, twice the warps).  A stage of 96 x 70 cells, 30 tiles: 0.178 ms
+// on two CTAs per SM, 0.169 on one, 0.137 on 16 x 8 tiles; of 512 x 512, 1024
+// tiles: 1.21 on one, 1.10 on two (before the inputs' prefetch).
 template <int QP, int QC, int STAGE>
 int launch_stage_2d(const DevParams& p, cudaStream_t s) {
-  const int ntx = (p.nx + Tile2::TX - 1) / Tile2::TX, nty = (p.ny + Tile2::TY - 1) / Tile2::TY;
+  const int ntx = (p.nx + 15) / 16;
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return (int)e;
-  const int ntiles = ntx * nty;
-  return ntiles <= nsm ? launch_stage_2d_c<QP, QC, STAGE, 1>(p, ntx, ntiles, nsm, s)
-                       : launch_stage_2d_c<QP, QC, STAGE, 2>(p, ntx, ntiles, nsm, s);
+  if (ntx * ((p.ny + 7) / 8) <= nsm) return launch_stage_2d_c<QP, QC, STAGE, 1, 8>(p, ntx, nsm, s);
+  if (ntx * ((p.ny + 15) / 16) <= nsm) return launch_stage_2d_c<QP, QC, STAGE, 1, 16>(p, ntx, nsm, s);
+  return launch_stage_2d_c<QP, QC, STAGE, 2, 16>(p, ntx, nsm, s);
 }
 
 template <int QP, int QC, int VAR>

@@ -332,11 +332,6 @@ __device__ __forceinline__ void mp9_march_fp32(const float* __restrict__ p, int 
   }
 }
 
-// Overloads so the stage kernel can march either storage type.
-template <int NSTEP>
-__device__ __forceinline__ void mp9_march(const double* p, int ss, double* out, int ostep) {
-  mp9_march_fp64<NSTEP>(p, ss, out, ostep);
-}
 template <int NSTEP>
 __device__ __forceinline__ void mp9_march(const float* p, int ss, float* out, int ostep) {
   mp9_march_fp32<NSTEP>(p, ss, out, ostep);

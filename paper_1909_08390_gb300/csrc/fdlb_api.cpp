@@ -339,6 +339,7 @@ void assign_buffers(fdlb_ctx* c, const Layout& L) {
   }
   c->mom = (double*)(b + L.mom);
   p.status = (unsigned*)(b + L.mom + 4 * (size_t)p.N * sizeof(double));
+  p.ticket = p.status + fdlb::kTicketWord;
 }
 
 // The mixed state to (out) or from the binary64 array x of P * N values.
@@ -354,7 +355,7 @@ double* mixed_exchange_buffer(fdlb_ctx* c) { return (double*)c->dp.r3l; }
 
 int ensure_prepared(fdlb_ctx* c) {
   if (c->prepared) return FDLB_OK;
-  cudaError_t me = cudaMemsetAsync(c->dp.status, 0, sizeof(unsigned), c->stream);
+  cudaError_t me = cudaMemsetAsync(c->dp.status, 0, (fdlb::kTicketWord + 1) * sizeof(unsigned), c->stream);
   if (me == cudaSuccess && c->batch)
     me = cudaMemsetAsync(c->dp.pstatus, 0, c->probs.size() * sizeof(unsigned), c->stream);
   if (me != cudaSuccess) return cuda_err(c, me, "status reset");

@@ -91,6 +91,7 @@ struct DevParams {
   void* Af;     // running explicit part of F^{n+1}
   void* D;      // F^n - F^n_eq
   unsigned* status;  // bit 0: invalid moments seen
+  unsigned* ticket;  // zero between launches: tiles handed out (2-D binary64)
   // batches of 1-D problems (nprob > 0): N is the total cell count
   const BatchProblem* probs;
   const WorkItem* work;
@@ -128,6 +129,9 @@ int batch_tile_cells(int variant);
 // kStateOut, kStateIn: the binary32-pair state of a FDLB_MIXED context to and
 // from the binary64 array xstate.
 enum Stage { kPrep = 0, kStage3 = 1, kStage4 = 2, kFinal = 3, kStateOut = 4, kStateIn = 5 };
+
+// The word of a context's 256-byte status block that holds the ticket.
+constexpr int kTicketWord = 32;
 
 // Kernel launchers (fdlb_kernels.cu).  Each returns a cudaError_t value.
 bool supported_lattice(int d, int Qp, int Qc);

@@ -260,15 +260,18 @@ struct Smem2 {
   AdvCoef coef[P];  // dt |p| / ds
   int cex[P];
   int ex[2][kG];
-  int mx[2][kG];    // largest magnitude words of the group's tiles
+  int mx[2][kG];  // magnitude words: the largest of the group's tiles,
+  int mn[2][kG];  // the smallest of their own cells
+  int next[2];    // the tile after this one, after the next one
 };
 
 // One fused stage.  Integer and binary64 work run side by side: 8 warps march
 // (staging, scaling and the fixed-point MP-9 flux differences: integer pipes)
 // one group of populations ahead of 8 warps that update (explicit parts,
 // moments and, per tile, pass 2: binary64 pipe), through two buffers of flux
-// differences.  The CTAs walk the tiles, so the march of the next tile runs
-// during pass 2.
+// differences.  Where a CTA has more than one tile, the march of the next one
+// runs during pass 2; it takes the tiles from a counter, because those that
+// march in binary64 (fdlb_mp9i.cuh) cost more.
 // Measured at 512 x 512 x 128 populations, per step: 9.93 ms with the march in
 // binary64 (that pipe 78 % busy), 3.64 ms with every warp marching and
 // updating in turn (the pipes idle in turn), 3.16 ms so.  What bounds it now:
@@ -286,10 +289,13 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
   extern __shared__ __align__(16) unsigned char smraw[];
   auto& sm = *reinterpret_cast<Smem2<QP, QC, TY_>*>(smraw);
   const int64_t N = p.N;
-  const int items = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x * GM::NG;
+  constexpr bool kMany = CTAS > 1;  // CTAs with more than one tile
   for (int pop = threadIdx.x; pop < L::P; pop += NM + NU)
     sm.coef[pop] = advection_coef(p.cx[pop], p.cy[pop], sm.cex[pop]);
-  if (threadIdx.x < 2 * kG) sm.mx[threadIdx.x / kG][threadIdx.x % kG] = 0;
+  if (threadIdx.x < 2 * kG) {
+    sm.mx[threadIdx.x / kG][threadIdx.x % kG] = 0;
+    sm.mn[threadIdx.x / kG][threadIdx.x % kG] = 0x7fffffff;
+  }
   __syncthreads();
 
   if (threadIdx.x < NM) {
@@ -309,7 +315,7 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
     // index clamp or wrap
     constexpr int NST = TY * (TX + 2 * H) + 2 * H * TX;
     constexpr int J = (NST + NM - 1) / NM;
-    int soff[J], goff[J];
+    int soff[J], goff[J], halo[J];  // halo: all ones, zero for the tile's own cells
     bool has[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
@@ -317,6 +323,7 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
       staged_pos(tid + j * NM, 2, TX, TY, r, c);
       has[j] = tid + j * NM < NST;
       soff[j] = r * T2::SX + c;
+      halo[j] = r >= H && r < H + TY && c >= H && c < H + TX ? 0 : 0x7fffffff;
     }
     auto set_tile = [&](int t) {
       const int x0 = t % ntx * TX, y0 = t / ntx * TY;
@@ -338,36 +345,60 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
         }
       cp_async_commit();
     };
-    int tile = blockIdx.x, gi = 0;
+    int tile = blockIdx.x, gi = 0, nth = 0;
+    bool more = true;
     set_tile(tile);
     prefetch(0, GM::first(0));
-    for (int it = 0; it < items; ++it) {
+    for (int it = 0; more; ++it) {
       const int b = it & 1, g0 = GM::first(gi);
-      // the scale of each population's tile: the largest magnitude
+      // the next tile's number; the last of the launch's ntiles requests leaves
+      // the counter as it was
+      if (kMany && gi == 0 && tid == 0) {
+        const unsigned k = atomicAdd(p.ticket, 1u);
+        if (k == (unsigned)ntiles - 1) *p.ticket = 0;
+        sm.next[nth & 1] = (int)(gridDim.x + k);
+      }
+      // each population's tile: the largest magnitude (its scale), and its own
+      // cells' smallest
       cp_async_wait_all();
+      int most = 0, least = 0;
 #pragma unroll
       for (int g = 0; g < kG; ++g) {
-        int m = 0;
+        int m = 0, l = 0x7fffffff;
 #pragma unroll
         for (int j = 0; j < J; ++j)
-          if (has[j]) m = max(m, mag_word(dfrom((&sm.tile[b][g][0][0])[soff[j]])));
-        m = (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
-        if (tid % 32 == g) atomicMax(&sm.mx[b][g], m);
+          if (has[j]) {
+            const int w = mag_word(dfrom((&sm.tile[b][g][0][0])[soff[j]]));
+            m = max(m, w);
+            l = min(l, w | halo[j]);
+          }
+        m = __reduce_max_sync(0xffffffffu, m);
+        l = __reduce_min_sync(0xffffffffu, l);
+        most = tid % 32 == g ? m : most;
+        least = tid % 32 == g ? l : least;
+      }
+      if (tid % 32 < kG) {
+        atomicMax(&sm.mx[b][tid % 32], most);
+        atomicMin(&sm.mn[b][tid % 32], least);
       }
       bar_sync(kMarchBar, NM);  // the magnitudes are in; the previous march is done
       int ngi = gi + 1;
       if (ngi == GM::NG) {
         ngi = 0;
-        tile += gridDim.x;
-        if (it + 1 < items) set_tile(tile);
+        tile = kMany ? sm.next[nth++ & 1] : ntiles;
+        more = tile < ntiles;
+        if (more) set_tile(tile);
       }
-      if (it + 1 < items) prefetch(b ^ 1, GM::first(ngi));
-      if (tid < kG) sm.mx[b ^ 1][tid] = 0;
+      if (more) prefetch(b ^ 1, GM::first(ngi));
+      if (tid < kG) {
+        sm.mx[b ^ 1][tid] = 0;
+        sm.mn[b ^ 1][tid] = 0x7fffffff;
+      }
       // cells to integers, once each and by the thread that copied them
 #pragma unroll
       for (int g = 0; g < kG; ++g) {
         const int emax = sm.mx[b][g] >> 20;
-        if (emax >= kQExpMin && emax <= kQExpMax) {
+        if (takes_fixed_point(sm.mx[b][g], sm.mn[b][g])) {
 #pragma unroll
           for (int j = 0; j < J; ++j)
             if (has[j]) {
@@ -387,7 +418,7 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
       const int64_t* up = line + (first - sgn) * step;
       int64_t* out = xline ? &sm.hx[b][tg][ln][first] : &sm.hy[b][tg][ln][first];
       const int emax = sm.mx[b][tg] >> 20;
-      const bool fixed = emax >= kQExpMin && emax <= kQExpMax;
+      const bool fixed = takes_fixed_point(sm.mx[b][tg], sm.mn[b][tg]);
       if (tid % PT == 0) sm.ex[b][tg] = fixed ? emax : 0;
       if (pop < L::P) {
         if (fixed) mp9_march_delta_int<T2::SEG>(up, sgn * step, out, sgn);
@@ -401,8 +432,8 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
     const int tid = threadIdx.x - NM;
     const int lx = tid % TX, ly = tid / TX;
     const Geo geo{p.nx, p.ny, 0, p.kchi, p.invDK, p.dtdx, p.dtdy, -1};
-    int it = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    int next = ntiles, nth = 0, it = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile = next, ++nth) {
       const int x = tile % ntx * TX + lx, y = tile / ntx * TY + ly;
       const bool valid = x < p.nx && y < p.ny;
       // (a thread without a cell reads the first one and stores nothing)
@@ -430,6 +461,7 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
           }
         }
         bar_sync(kFull + b, NM + NU);  // the group's flux differences are in
+        if (kMany && gi == 0) next = sm.next[nth & 1];
         double R[kG];
 #pragma unroll
         for (int g = 0; g < kG; ++g) {
@@ -444,7 +476,8 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
             R[g] = store_update<STAGE>(p, pop * N, c, valid, in[g], X);
           }
         }
-        if (it + 2 < items) bar_arrive(kEmpty + b, NM + NU);
+        // (the march waits for it two groups on, if it gets there)
+        if (gi + 2 < GM::NG || next < ntiles) bar_arrive(kEmpty + b, NM + NU);
         mom.add(p, g0, R);
         mom.fold(p, gi);
       }

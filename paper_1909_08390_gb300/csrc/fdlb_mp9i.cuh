@@ -1,24 +1,40 @@
 // fdlb_mp9i.cuh -- the MP-9 march of fdlb_mp9.cuh (Sec. IV) in 64-bit
-// fixed point, for the binary64 stage kernels.
+// fixed point, for the 2-D binary64 stage kernels.
 //
 // GB300 runs 2 binary64 operations per clock and SM, but 64 integer
 // operations (shifts, logic, compares, 32 x 32 -> 64 multiply-adds) and about
 // 128 integer additions.  The march is a fixed sequence of differences, one
 // stencil with integer coefficients and a limiter made of comparisons, so it
-// needs no exponents inside a line: the cells of a line (or, in 1-D, of a
-// block of 8 cells) and its 5-cell halo are scaled to integers
+// needs no exponents as long as its values are of similar size: a population's
+// cells of one tile with their 5-cell halo are scaled to integers
 //   q = F 2^(59 - E),  2^E > max |F| of those cells,
-// truncated at one unit.  A unit is 2^-59 of the largest value, 1/64 of its
-// binary64 rounding unit; differences, curvatures and flux differences are
-// then exact, the stencil and the limiter's bounds lose at most two units
-// each, and the flux difference of a cell goes back to binary64 with one
-// rounding.  (The binary64 march rounds every interface value to 2^-53 of
-// itself.)  Sizes: |q| < 2^59, differences < 2^60, curvatures < 2^61,
-// 4 m - M <= 3 m < 2^62.6, bounds < 2^62: all inside 63 bits.
+// truncated at one unit.  A unit is 2^-59 of the largest value's power of two;
+// differences, curvatures and flux differences are then exact, the stencil and
+// the limiter's bounds lose at most two units each, and the flux difference of
+// a cell goes back to binary64 with one rounding.  Sizes: |q| < 2^59,
+// differences < 2^60, curvatures < 2^61, 4 m - M <= 3 m < 2^62.6, bounds <
+// 2^62: all inside 63 bits.
 //
-// Lines whose largest exponent leaves no room for the scaling (an infinity or
-// NaN among the cells, values beyond 2^1007 or below 2^-823) march in
-// binary64 (mp9_march_delta_fp64).
+// So the error is relative to the tile's largest value, where the binary64
+// march rounds every interface value to 2^-53 of itself: the smaller a cell
+// beside the tile's largest, the less the fixed-point march is worth.  Root
+// mean square error of a flux difference over its cell's own value, smooth
+// lines | rough ones (uniform within 50 %), for cells r times below the
+// largest, against 7e-17 | 4.5e-17 in binary64:
+//   r = 1 2e-18 | 6e-18,  4 5e-18 | 1.2e-17,  16 2e-17 | 4.4e-17,
+//   32 4e-17 | 8e-17,  64 1e-16 | 1.6e-16.
+// Hence the rule (takes_fixed_point): a tile whose own cells lie no more than a
+// factor of 16 below the largest of tile and halo, so that no cell's error is
+// larger than in binary64 (root mean square).  The others, tiles with a zero
+// among nonzero cells, and those whose largest exponent leaves no room for the
+// scaling (an infinity or NaN among the cells, values beyond 2^1007 or below
+// 2^-823), march in binary64 (mp9_march_delta_fp64).
+//
+// The scale and the choice belong to the tile, so the last bits of a result
+// depend on where the tiles lie: a periodic field shifted by other than whole
+// tiles, or run on a device with another number of SMs (which sets the tile
+// height of small grids), differs by roundings, and an interface on a tile's
+// edge, computed once on either side, cancels to rounding only.
 //
 // The flux differences stay integers until the update of a cell: the
 // advection term dt p . grad F is their sum times 61-bit fixed-point
@@ -35,8 +51,10 @@
 namespace fdlb {
 
 constexpr int kQBits = 59;  // |q| < 2^kQBits
-// biased exponents of the line's largest magnitude that the march takes
+// biased exponents of the cells' largest magnitude that the march takes
 constexpr int kQExpMin = 200, kQExpMax = 2030;
+// and the distance of its magnitude word from the smallest one's: 2^4
+constexpr int kQRange = 4 << 20;
 
 // x >> n for any n >= 0 (zero from 64 on)
 __device__ __forceinline__ uint64_t shr64(uint64_t x, int n) {
@@ -58,6 +76,13 @@ __device__ __forceinline__ int clz64(uint64_t x) {
 
 // high word of |x|: its biased exponent is bits 20..30; ordered like |x|
 __device__ __forceinline__ int mag_word(double x) { return (int)(dbits(x) >> 32) & 0x7fffffff; }
+// Whether the fixed-point march takes cells whose largest magnitude word is mx
+// and whose flux differences are wanted down to magnitude word mn (see the head
+// of this file).
+__device__ __forceinline__ bool takes_fixed_point(int mx, int mn) {
+  const int e = mx >> 20;
+  return e >= kQExpMin && e <= kQExpMax && mx - mn <= kQRange;
+}
 
 // x as a fixed-point integer of a line whose largest biased exponent is emax
 __device__ __forceinline__ int64_t q_of(double x, int emax) {
@@ -270,17 +295,39 @@ __device__ __forceinline__ void mp9_march_delta_int(const int64_t* __restrict__ 
 #undef FDLB_STEP
 }
 
-// The same flux differences in binary64 (their bits), for lines the
-// fixed-point march does not take; one interface at a time (rare: kept small).
+// The same flux differences in binary64 (their bits), for tiles the
+// fixed-point march does not take.  The window slides (15 binary64 operations
+// an interface) in a loop that isn't unrolled (kept small).
 __device__ __noinline__ void mp9_march_delta_fp64(const double* p, int ss, int64_t* out, int ostep,
                                                   int nc) {
+  Mp9Line L;
+  double v = p[-4 * ss];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const double x = p[(k - 3) * ss];
+    L.d[k] = x - v;
+    v = x;
+  }
+  L.c0 = L.d[4] - L.d[3];
+  L.dmm = dm_bits(L.d[3] - L.d[2], L.c0);
   double prev = 0.0;
 #pragma unroll 1
   for (int t = 0; t <= nc; ++t) {
-    double f;
-    mp9_march_fp64<1>(p + t * ss, ss, &f, 1);
+    double c1;
+    long long dmp;
+    L.fs[0] = p[t * ss];
+    const double f = mp9_face_fp64(L, c1, dmp);
     if (t > 0) out[(t - 1) * ostep] = dbits(f - prev);
     prev = f;
+    if (t < nc) {
+      const double x = p[(t + 5) * ss];
+#pragma unroll
+      for (int k = 0; k < 7; ++k) L.d[k] = L.d[k + 1];
+      L.d[7] = x - v;
+      v = x;
+      L.c0 = c1;
+      L.dmm = dmp;
+    }
   }
 }
 

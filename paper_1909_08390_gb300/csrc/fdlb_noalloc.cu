@@ -81,9 +81,10 @@ extern "C" int fdlb_step_noalloc(const fdlb_grid* grid, int Qphi, int Qchi, doub
   p.D = (double*)(b + 4 * arr);
   p.status = (unsigned*)(b + 5 * arr);
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  // the status word must start at zero; every other scratch element is
+  p.ticket = p.status + fdlb::kTicketWord;
+  // the status word and the ticket must start at zero; every other scratch element is
   // written before it is read
-  cudaError_t e = cudaMemsetAsync(p.status, 0, sizeof(unsigned), s);
+  cudaError_t e = cudaMemsetAsync(p.status, 0, kStatusBytes, s);
   if (e != cudaSuccess) return cuda_fail(e);
   int le = fdlb::launch_stage(p, fdlb::kPrep, s);
   for (int64_t k = 0; k < nsteps && !le; ++k)

@@ -771,7 +771,7 @@ __device__ __forceinline__ int find_problem(const DevParams& p, int64_t c) {
 }
 
 // D and F2 of a state that was set (fdlb_init_riemann, fdlb_set_state), one
-// cell per thread.
+// cell per thread, by the final stage's operations in their order.
 template <int DIM, int QP, int QC>
 __global__ void __launch_bounds__(128) prep_kernel(const __grid_constant__ DevParams p) {
   __shared__ double fac[DIM == 2 ? QP + QC : 1][128];
@@ -784,8 +784,25 @@ __global__ void __launch_bounds__(128) prep_kernel(const __grid_constant__ DevPa
     geo.invDK = p.probs[geo.prob].invDK;
   }
   Moments m = {};
-  for (int pop = 0; pop < Lat<DIM, QP, QC>::P; ++pop)
-    accumulate<DIM, QP, QC>(p, m, pop, ((const double*)p.F + pop * p.N)[c]);
+  if constexpr (DIM == 2) {
+    // in the final stage's order, so that a run set from its own populations
+    // goes on with the same bits
+    using GM = GroupMoments<QP, QC>;
+    GM g = {};
+#pragma unroll 2
+    for (int gi = 0; gi < GM::NG; ++gi) {
+      const int g0 = GM::first(gi);
+      double v[kG];
+#pragma unroll
+      for (int j = 0; j < kG; ++j) v[j] = g0 + j < GM::P ? ((const double*)p.F + (g0 + j) * p.N)[c] : 0.0;
+      g.add(p, g0, v);
+      g.fold(p, gi);
+    }
+    m = g.m;
+  } else {
+    for (int pop = 0; pop < Lat<DIM, QP, QC>::P; ++pop)
+      accumulate<DIM, QP, QC>(p, m, pop, ((const double*)p.F + pop * p.N)[c]);
+  }
   relax_cell64<DIM, QP, QC, kPrep, 128>(p, geo, (unsigned)c, m, &fac[0][threadIdx.x]);
 }
 

@@ -39,11 +39,11 @@ template <int DIM, int QP, int QC, int STAGE, int FS>
 __device__ __forceinline__ void relax_cell64(const DevParams& p, const Geo& geo, unsigned c,
                                              const Moments& m, double* fac) {
   const int64_t N = p.N;
-  const double* __restrict__ const Rin =
+  // (stages 3 and 4 relax in place: Rin and Fout are one array there)
+  const double* const Rin =
       (const double*)(STAGE == kStage3 ? p.F3 : STAGE == kStage4 ? p.A4 : p.F);
-  double* __restrict__ const Fout =
-      (double*)(STAGE == kStage3 ? p.F3 : STAGE == kStage4 ? p.A4 : p.F2);
-  double* __restrict__ const Dn = (double*)p.D;
+  double* const Fout = (double*)(STAGE == kStage3 ? p.F3 : STAGE == kStage4 ? p.A4 : p.F2);
+  double* const Dn = (double*)p.D;
   const StageCoef& sc = p.sc;
   const double kd = STAGE == kStage3 ? sc.a33e3 : STAGE == kStage4 ? sc.a44e4 : sc.c2m1;
   constexpr int W = QP > QC ? QP : QC;

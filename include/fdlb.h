@@ -121,7 +121,10 @@ int fdlb_named_tableau(int which, fdlb_tableau* out);
  *                high part; per-cell moment sums are binary64, so n, u, T
  *                (including the cancellation in T = (E - n u^2)/((D+K) n))
  *                are binary64, and the equilibrium factors are binary32
- *                pairs
+ *                pairs.  A 2-D grid's arrays have both sides rounded up to
+ *                multiples of 16 cells where that takes at most an eighth
+ *                or 32768 cells more, or, up to 2^18 cells so rounded, at
+ *                most twice the cells
  *   cuda_stream: cudaStream_t to enqueue on (NULL: the legacy default stream)
  *   out        : receives the context (NULL on failure)
  * The populations start at zero; call fdlb_init_riemann or fdlb_set_state. */

@@ -15,6 +15,7 @@
 #include "fdlb.h"
 #include "fdlb_ctx.h"
 #include "fdlb_internal.h"
+#include "fdlb_tile.cuh"
 
 using fdlb::DevParams;
 using fdlb::kMaxQ;
@@ -286,15 +287,13 @@ struct Layout {
 };
 
 // Row pitch and population stride of a context's arrays (DevParams::pitch).
-// FDLB_MIXED 2-D grids are padded to whole tiles unless they are so thin that
-// the padding would cost more than an eighth and more than 2^18 cells.
 void set_strides(DevParams& p) {
   p.pitch = p.nx;
   p.padded = 0;
   p.NS = p.N;
   if (p.precision != FDLB_MIXED || p.d != 2) return;
+  if (!fdlb::pads_to_tiles(p.nx, p.ny)) return;
   const int64_t px = ((int64_t)p.nx + 15) / 16 * 16, py = ((int64_t)p.ny + 15) / 16 * 16;
-  if (px * py > (1 << 18) && 8 * px * py > 9 * p.N) return;
   p.pitch = (int)px;
   p.padded = 1;
   p.NS = px * py;

@@ -62,15 +62,6 @@ inline int single_1d_variant(int64_t nx) {
   if (nx >= 31 * 152) return 4;
   return 3;
 }
-inline int tile_cells_1d(int variant) {
-  switch (variant) {
-    case 1: return TileCfg<1, 1>::TX;
-    case 2: return TileCfg<1, 2>::TX;
-    case 3: return TileCfg<1, 3>::TX;
-    case 4: return TileCfg<1, 4>::TX;
-    default: return TileCfg<1, 0>::TX;
-  }
-}
 
 // Where a tile lives: its problem's size, first cell in the population
 // arrays, and gas and grid constants.
@@ -189,11 +180,6 @@ __device__ __forceinline__ bool moments_to_nut(double invDK, const Moments& m, d
   return (n > 0.0) && (T > 0.0) && isfinite(n) && isfinite(T) && isfinite(ux) && isfinite(uy);
 }
 
-// ---- storage-type helpers --------------------------------------------------
-
-__device__ __forceinline__ double sfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float sfma(float a, float b, float c) { return fmaf(a, b, c); }
-
 // Moment sums of binary32 populations, kept as unevaluated binary32 pairs
 // (hi + lo) with error-free transformations: TwoSum for each addition and the
 // fma-exact product error for p * v with p = hi + lo split on the host.  The
@@ -276,22 +262,10 @@ __device__ __forceinline__ MomentsF lane(const MomentsF2& m, int i) {
   return MomentsF{g(m.nh), g(m.nl), g(m.jxh), g(m.jxl), g(m.jyh), g(m.jyl), g(m.eh), g(m.el)};
 }
 
-__device__ __forceinline__ Moments to_fp64(const Moments& m) { return m; }
 __device__ __forceinline__ Moments to_fp64(const MomentsF& m) {
   return Moments{(double)m.nh + (double)m.nl, (double)m.jxh + (double)m.jxl,
                  (double)m.jyh + (double)m.jyl, (double)m.eh + (double)m.el};
 }
-
-template <typename S>
-struct MomAcc;
-template <>
-struct MomAcc<double> {
-  using type = Moments;
-};
-template <>
-struct MomAcc<float> {
-  using type = MomentsF;
-};
 
 // Equilibrium factors in the storage type (binary32 copies of the binary64
 // per-cell factors on the mixed path).

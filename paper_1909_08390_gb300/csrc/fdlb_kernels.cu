@@ -936,19 +936,19 @@ __global__ void mixed_moments_kernel(const __grid_constant__ DevParams p, double
   T[c] = TT;
 }
 
-template <int DIM, int QP, int QC, typename S>
+template <int DIM, int QP, int QC>
 __global__ void moments_kernel(const __grid_constant__ DevParams p, double* __restrict__ n,
                                double* __restrict__ ux, double* __restrict__ uy,
                                double* __restrict__ T) {
   using L = Lat<DIM, QP, QC>;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= p.N) return;
-  typename MomAcc<S>::type m = {};
-  const S* F = (const S*)p.F;
+  Moments m = {};
+  const double* F = (const double*)p.F;
   for (int pop = 0; pop < L::P; ++pop) accumulate<DIM, QP, QC>(p, m, pop, F[pop * p.N + c]);
   double nn, vx, vy, TT;
   const double invDK = p.nprob > 0 ? p.probs[find_problem(p, c)].invDK : p.invDK;
-  moments_to_nut<DIM>(invDK, to_fp64(m), nn, vx, vy, TT);
+  moments_to_nut<DIM>(invDK, m, nn, vx, vy, TT);
   n[c] = nn;
   ux[c] = vx;
   if (DIM == 2 && uy) uy[c] = vy;
@@ -1100,7 +1100,7 @@ int launch_moments_t(const DevParams& p, double* n, double* ux, double* uy, doub
   const int nt = 128;
   const int64_t nb = (p.N + nt - 1) / nt;
   if (p.precision == 1) mixed_moments_kernel<DIM, QP, QC><<<(unsigned)nb, nt, 0, s>>>(p, n, ux, uy, T);
-  else moments_kernel<DIM, QP, QC, double><<<(unsigned)nb, nt, 0, s>>>(p, n, ux, uy, T);
+  else moments_kernel<DIM, QP, QC><<<(unsigned)nb, nt, 0, s>>>(p, n, ux, uy, T);
   return (int)cudaGetLastError();
 }
 

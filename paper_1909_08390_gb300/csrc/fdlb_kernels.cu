@@ -251,18 +251,17 @@ template <int QP, int QC, int TY>
 struct Smem2 {
   using T2 = Tile2<TY>;
   static constexpr int P = Lat<2, QP, QC>::P;
-  int64_t tile[2][kG][T2::SY][T2::SX];  // cells + halo: binary64, then integers
-  // flux differences along x and y, in units of the scale with exponent ex
-  // (0: binary64 bits)
+  double tile[2][kG][T2::SY][T2::SX];  // cells + halo
+  // flux differences along x and y, in units of their half line's scale, whose
+  // exponents are in ex and ey (0: binary64 bits)
   int64_t hx[2][kG][T2::TY][T2::TX + 1];
   int64_t hy[2][kG][T2::TX][T2::TY + 1];
+  int ex[2][kG][T2::TY][T2::TX / T2::SEG];
+  int ey[2][kG][T2::TX][T2::TY / T2::SEG];
   double fac[QP + (QC == QP ? 0 : QC)][T2::NU];
   AdvCoef coef[P];  // dt |p| / ds
   int cex[P];
-  int ex[2][kG];
-  int mx[2][kG];  // magnitude words: the largest of the group's tiles,
-  int mn[2][kG];  // the smallest of their own cells
-  int next[2];    // the tile after this one, after the next one
+  int next[2];  // the tile after this one, after the next one
 };
 
 // One fused stage.  Integer and binary64 work run side by side: 8 warps march
@@ -270,14 +269,17 @@ struct Smem2 {
 // one group of populations ahead of 8 warps that update (explicit parts,
 // moments and, per tile, pass 2: binary64 pipe), through two buffers of flux
 // differences.  Where a CTA has more than one tile, the march of the next one
-// runs during pass 2; it takes the tiles from a counter, because those that
-// march in binary64 (fdlb_mp9i.cuh) cost more.
-// Measured at 512 x 512 x 128 populations, per step: 9.93 ms with the march in
-// binary64 (that pipe 78 % busy), 3.64 ms with every warp marching and
-// updating in turn (the pipes idle in turn), 3.16 ms so.  What bounds it now:
-// about 680 instructions per population-cell and stage at half the issue
-// rate, the integer pipe and the binary64 pipe each about half busy; 16 warps
-// a CTA wait on the fixed latency of 64-bit integer chains.
+// runs during pass 2; it takes the tiles from a counter, because those with
+// lines that march in binary64 (fdlb_mp9i.cuh) cost more.
+// Measured at 512 x 512 x 128 populations, a step: 9.93 ms with every tile
+// marching in binary64 and every warp marching and updating in turn (that pipe
+// 78 % busy); 3.36 ms for a smooth field, all in fixed point; 3.87 ms for four
+// quadrants, where 6 % of the groups have a line in binary64.  What bounds it:
+// about 700 instructions per population-cell and stage at half the issue rate,
+// the integer pipe and the binary64 pipe each about half busy; 16 warps a CTA
+// wait on the fixed latency of 64-bit integer chains.  A line in binary64 is a
+// chain of 145 instructions of 64 cycles, about as long again as a group, and
+// the last tiles with such lines run beside idle SMs.
 template <int QP, int QC, int STAGE, int CTAS, int TY_>
 __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
     stage_kernel_2d(const __grid_constant__ DevParams p, int ntx, int ntiles) {
@@ -292,10 +294,6 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
   constexpr bool kMany = CTAS > 1;  // CTAs with more than one tile
   for (int pop = threadIdx.x; pop < L::P; pop += NM + NU)
     sm.coef[pop] = advection_coef(p.cx[pop], p.cy[pop], sm.cex[pop]);
-  if (threadIdx.x < 2 * kG) {
-    sm.mx[threadIdx.x / kG][threadIdx.x % kG] = 0;
-    sm.mn[threadIdx.x / kG][threadIdx.x % kG] = 0x7fffffff;
-  }
   __syncthreads();
 
   if (threadIdx.x < NM) {
@@ -315,7 +313,7 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
     // index clamp or wrap
     constexpr int NST = TY * (TX + 2 * H) + 2 * H * TX;
     constexpr int J = (NST + NM - 1) / NM;
-    int soff[J], goff[J], halo[J];  // halo: all ones, zero for the tile's own cells
+    int soff[J], goff[J];
     bool has[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
@@ -323,7 +321,6 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
       staged_pos(tid + j * NM, 2, TX, TY, r, c);
       has[j] = tid + j * NM < NST;
       soff[j] = r * T2::SX + c;
-      halo[j] = r >= H && r < H + TY && c >= H && c < H + TX ? 0 : 0x7fffffff;
     }
     auto set_tile = [&](int t) {
       const int x0 = t % ntx * TX, y0 = t / ntx * TY;
@@ -341,7 +338,7 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
           const double* __restrict__ src = adv + (g0 + g) * N;
 #pragma unroll
           for (int j = 0; j < J; ++j)
-            if (has[j]) cp_async((double*)&sm.tile[b][g][0][0] + soff[j], src + (unsigned)goff[j]);
+            if (has[j]) cp_async(&sm.tile[b][g][0][0] + soff[j], src + (unsigned)goff[j]);
         }
       cp_async_commit();
     };
@@ -358,30 +355,8 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
         if (k == (unsigned)ntiles - 1) *p.ticket = 0;
         sm.next[nth & 1] = (int)(gridDim.x + k);
       }
-      // each population's tile: the largest magnitude (its scale), and its own
-      // cells' smallest
       cp_async_wait_all();
-      int most = 0, least = 0;
-#pragma unroll
-      for (int g = 0; g < kG; ++g) {
-        int m = 0, l = 0x7fffffff;
-#pragma unroll
-        for (int j = 0; j < J; ++j)
-          if (has[j]) {
-            const int w = mag_word(dfrom((&sm.tile[b][g][0][0])[soff[j]]));
-            m = max(m, w);
-            l = min(l, w | halo[j]);
-          }
-        m = __reduce_max_sync(0xffffffffu, m);
-        l = __reduce_min_sync(0xffffffffu, l);
-        most = tid % 32 == g ? m : most;
-        least = tid % 32 == g ? l : least;
-      }
-      if (tid % 32 < kG) {
-        atomicMax(&sm.mx[b][tid % 32], most);
-        atomicMin(&sm.mn[b][tid % 32], least);
-      }
-      bar_sync(kMarchBar, NM);  // the magnitudes are in; the previous march is done
+      bar_sync(kMarchBar, NM);  // the group's tile is in; the previous march is done
       int ngi = gi + 1;
       if (ngi == GM::NG) {
         ngi = 0;
@@ -390,39 +365,22 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
         if (more) set_tile(tile);
       }
       if (more) prefetch(b ^ 1, GM::first(ngi));
-      if (tid < kG) {
-        sm.mx[b ^ 1][tid] = 0;
-        sm.mn[b ^ 1][tid] = 0x7fffffff;
-      }
-      // cells to integers, once each and by the thread that copied them
-#pragma unroll
-      for (int g = 0; g < kG; ++g) {
-        const int emax = sm.mx[b][g] >> 20;
-        if (takes_fixed_point(sm.mx[b][g], sm.mn[b][g])) {
-#pragma unroll
-          for (int j = 0; j < J; ++j)
-            if (has[j]) {
-              int64_t& v = (&sm.tile[b][g][0][0])[soff[j]];
-              v = q_of(dfrom(v), emax);
-            }
-        }
-      }
-      bar_sync(kMarchBar, NM);  // the group's tile is in
       if (it >= 2) bar_sync(kEmpty + b, NM + NU);  // the update is done with this buffer
       const int pop = g0 + tg;
       const double pv = pop < L::P ? (xline ? p.px[pop] : p.py[pop]) : 0.0;
       const int sgn = pv >= 0.0 ? 1 : -1;
       const int first = sgn > 0 ? s0 : s0 + T2::SEG - 1;
       const int step = xline ? 1 : T2::SX;
-      const int64_t* line = xline ? &sm.tile[b][tg][ln + H][H] : &sm.tile[b][tg][H][ln + H];
-      const int64_t* up = line + (first - sgn) * step;
+      const double* line = xline ? &sm.tile[b][tg][ln + H][H] : &sm.tile[b][tg][H][ln + H];
+      const double* up = line + (first - sgn) * step;
       int64_t* out = xline ? &sm.hx[b][tg][ln][first] : &sm.hy[b][tg][ln][first];
-      const int emax = sm.mx[b][tg] >> 20;
-      const bool fixed = takes_fixed_point(sm.mx[b][tg], sm.mn[b][tg]);
-      if (tid % PT == 0) sm.ex[b][tg] = fixed ? emax : 0;
       if (pop < L::P) {
-        if (fixed) mp9_march_delta_int<T2::SEG>(up, sgn * step, out, sgn);
-        else mp9_march_delta_fp64((const double*)up, sgn * step, out, sgn, T2::SEG);
+        // (a warp's lines, of one population, march either way as a whole)
+        int emax;
+        const bool fixed = __all_sync(0xffffffffu, scale_of_line<T2::SEG>(up, sgn * step, emax));
+        (xline ? sm.ex[b][tg][ln] : sm.ey[b][tg][ln])[s0 / T2::SEG] = fixed ? emax : 0;
+        if (fixed) mp9_march_delta<T2::SEG>(ScaledCells{up, emax}, sgn * step, out, sgn);
+        else mp9_march_delta_fp64(up, sgn * step, out, sgn, T2::SEG);
       }
       bar_arrive(kFull + b, NM + NU);
       gi = ngi;
@@ -450,7 +408,7 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
         load(g0, in);
         // the next group's inputs on their way to L2, a thread per tile row,
         // population and array: the registers to load them ahead are not there
-        // (512 x 512: 3.28 -> 3.16 ms a step; grids of few tiles sit in L2)
+        // (512 x 512: 3.42 -> 3.36 ms a step; grids of few tiles sit in L2)
         if (CTAS == 2 && TY == 16 && gi + 1 < GM::NG && tid < (STAGE == kStage4 ? 3 : 2) * 16 * kG) {
           const int row = tid % 16, pop = GM::first(gi + 1) + tid / 16 % kG, arr = tid / (16 * kG);
           const int xr = tile % ntx * TX, yr = tile / ntx * TY + row;
@@ -470,9 +428,10 @@ __global__ void __launch_bounds__(Tile2<TY_>::NM + Tile2<TY_>::NU, CTAS)
           if (pop < L::P) {
             // X = dt p . grad F
             const int64_t dx = sm.hx[b][g][ly][lx], dy = sm.hy[b][g][lx][ly];
-            const int ex = sm.ex[b][g];
-            double X = q_to_double(advection_int(sm.coef[pop], dx, dy), ex + sm.cex[pop]);
-            if (!ex) X = advection_bits(p.cx[pop], p.cy[pop], dx, dy);
+            const int ex = sm.ex[b][g][ly][lx / T2::SEG], ey = sm.ey[b][g][lx][ly / T2::SEG];
+            const int e = max(ex, ey);
+            double X = q_to_double(advection_int(sm.coef[pop], sar64(dx, e - ex), sar64(dy, e - ey)), e + sm.cex[pop]);
+            if (!ex || !ey) X = advection_fp64(p.cx[pop], p.cy[pop], dx, ex, dy, ey);
             R[g] = store_update<STAGE>(p, pop * N, c, valid, in[g], X);
           }
         }
@@ -1018,9 +977,10 @@ int launch_stage_2d_c(const DevParams& p, int ntx, int nsm, cudaStream_t s) {
 // Grids of no more tiles than SMs run one CTA per SM, whose threads then have
 // 128 registers, on tiles of 16 x 8 cells while these too have an SM each (a
 // stage's time is then one tile's); larger grids run two CTAs of 64 registers
-// (some spills, twice the warps).  A stage of 96 x 70 cells, 30 tiles: 0.178 ms
-// on two CTAs per SM, 0.169 on one, 0.137 on 16 x 8 tiles; of 512 x 512, 1024
-// tiles: 1.21 on one, 1.10 on two (before the inputs' prefetch).
+// (some spills, twice the warps).  A stage of 96 x 70 cells, 30 tiles, smooth
+// field | quadrants: 0.187 | 0.356 ms on two CTAs per SM, 0.153 | 0.348 on one,
+// 0.110 | 0.254 on 16 x 8 tiles; of 512 x 512, 1024 tiles: 1.10 | 1.30 on one,
+// 1.12 | 1.29 on two.
 template <int QP, int QC, int STAGE>
 int launch_stage_2d(const DevParams& p, cudaStream_t s) {
   const int ntx = (p.nx + 15) / 16;

@@ -5,9 +5,10 @@
 // operations (shifts, logic, compares, 32 x 32 -> 64 multiply-adds) and about
 // 128 integer additions.  The march is a fixed sequence of differences, one
 // stencil with integer coefficients and a limiter made of comparisons, so it
-// needs no exponents as long as its values are of similar size: a population's
-// cells of one tile with their 5-cell halo are scaled to integers
-//   q = F 2^(59 - E),  2^E > max |F| of those cells,
+// needs no exponents as long as its values are of similar size: the 17 values
+// that a marching thread reads for the 8 cells of its half line are scaled to
+// integers
+//   q = F 2^(59 - E),  2^E > max |F| of those values,
 // truncated at one unit.  A unit is 2^-59 of the largest value's power of two;
 // differences, curvatures and flux differences are then exact, the stencil and
 // the limiter's bounds lose at most two units each, and the flux difference of
@@ -15,26 +16,33 @@
 // differences < 2^60, curvatures < 2^61, 4 m - M <= 3 m < 2^62.6, bounds <
 // 2^62: all inside 63 bits.
 //
-// So the error is relative to the tile's largest value, where the binary64
+// So the error is relative to the largest of these values, where the binary64
 // march rounds every interface value to 2^-53 of itself: the smaller a cell
-// beside the tile's largest, the less the fixed-point march is worth.  Root
-// mean square error of a flux difference over its cell's own value, smooth
-// lines | rough ones (uniform within 50 %), for cells r times below the
-// largest, against 7e-17 | 4.5e-17 in binary64:
+// beside the largest, the less the fixed-point march is worth.  Root mean
+// square error of a flux difference over its cell's own value, smooth lines |
+// rough ones (uniform within 50 %), for cells r times below the largest,
+// against 7e-17 | 4.5e-17 in binary64:
 //   r = 1 2e-18 | 6e-18,  4 5e-18 | 1.2e-17,  16 2e-17 | 4.4e-17,
 //   32 4e-17 | 8e-17,  64 1e-16 | 1.6e-16.
-// Hence the rule (takes_fixed_point): a tile whose own cells lie no more than a
-// factor of 16 below the largest of tile and halo, so that no cell's error is
-// larger than in binary64 (root mean square).  The others, tiles with a zero
+// Hence the rule (takes_fixed_point): a half line whose own cells lie no more
+// than a factor of 16 below the largest value read, so that no cell's error is
+// larger than in binary64 (root mean square).  The others, lines with a zero
 // among nonzero cells, and those whose largest exponent leaves no room for the
-// scaling (an infinity or NaN among the cells, values beyond 2^1007 or below
-// 2^-823), march in binary64 (mp9_march_delta_fp64).
+// scaling (an infinity or NaN among the values, beyond 2^1007 or below 2^-823),
+// march in binary64 (mp9_march_delta_fp64), with the other lines of their warp.
 //
-// The scale and the choice belong to the tile, so the last bits of a result
-// depend on where the tiles lie: a periodic field shifted by other than whole
-// tiles, or run on a device with another number of SMs (which sets the tile
-// height of small grids), differs by roundings, and an interface on a tile's
-// edge, computed once on either side, cancels to rounding only.
+// One scale for a population's whole tile needs a conversion per cell instead
+// of two, but sends whole tiles to the binary64 march where a smooth field
+// varies by more than 16 over 26 cells.  512 x 512 x 128 populations, a step,
+// tile's scale -> line's: smooth field 3.05 -> 3.36 ms, four quadrants 3.89 ->
+// 3.87; 400 x 400 quadrants 3.23 -> 2.95; 96 x 70, smooth 0.405 -> 0.324,
+// quadrants 0.824 -> 0.760.
+//
+// The scales belong to half lines and the choice to warps, so the last bits of
+// a result depend on where the tiles lie: a periodic field shifted by other than
+// whole tiles, or run on a device with another number of SMs (which sets the
+// tile height of small grids), differs by roundings, and an interface on the
+// edge of a half line, computed once on either side, cancels to rounding only.
 //
 // The flux differences stay integers until the update of a cell: the
 // advection term dt p . grad F is their sum times 61-bit fixed-point
@@ -66,6 +74,16 @@ __device__ __forceinline__ uint64_t shr64(uint64_t x, int n) {
   return n > 63 ? 0 : x >> n;
 #endif
 }
+// x >> n (arithmetic) for any n >= 0
+__device__ __forceinline__ int64_t sar64(int64_t x, int n) {
+#ifdef __CUDA_ARCH__
+  int64_t r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));  // clamps n
+  return r;
+#else
+  return x >> (n > 63 ? 63 : n);
+#endif
+}
 __device__ __forceinline__ int clz64(uint64_t x) {
 #ifdef __CUDA_ARCH__
   return __clzll((long long)x);
@@ -84,7 +102,7 @@ __device__ __forceinline__ bool takes_fixed_point(int mx, int mn) {
   return e >= kQExpMin && e <= kQExpMax && mx - mn <= kQRange;
 }
 
-// x as a fixed-point integer of a line whose largest biased exponent is emax
+// x as a fixed-point integer of the scale whose largest biased exponent is emax
 __device__ __forceinline__ int64_t q_of(double x, int emax) {
   const long long b = dbits(x);
   const int hi = (int)(b >> 32);
@@ -224,8 +242,21 @@ __device__ __forceinline__ int64_t mp9_offset_int(const Mp9Int& L, int64_t& c1, 
 #undef FDLB_D
 }
 
+// The cells of a line as integers: stored so, or binary64 values scaled as
+// they're read.
+struct IntCells {
+  const int64_t* p;
+  __device__ __forceinline__ int64_t operator[](int i) const { return p[i]; }
+};
+struct ScaledCells {
+  const double* p;
+  int emax;
+  __device__ __forceinline__ int64_t operator[](int i) const { return q_of(p[i], emax); }
+};
+
 // The window of the first interface: F_{s-4}..F_{s+4} at p[(j - 4) ss].
-__device__ __forceinline__ void mp9_start_int(Mp9Int& L, const int64_t* p, int ss) {
+template <typename Cells>
+__device__ __forceinline__ void mp9_start_int(Mp9Int& L, const Cells& p, int ss) {
   int64_t v = p[-4 * ss];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
@@ -261,13 +292,12 @@ __device__ __forceinline__ int64_t mp9_step_int(Mp9Int& L, int64_t vnew, bool mo
 
 // March the NC + 1 interfaces around NC cells (NC a multiple of 8, or less
 // than 8) upwind to downwind and write each cell's flux difference
-// sgn (Fhat_right - Fhat_left) = d_-1 + a_cur - a_prev, in units of the line,
+// sgn (Fhat_right - Fhat_left) = d_-1 + a_cur - a_prev, in units of the scale,
 // at out[t * ostep] (|.| < 2^62.4: two offsets below 2^61 and a difference); `p`
 // points at the upwind cell of the first interface, ss is the signed element
 // stride.
-template <int NC>
-__device__ __forceinline__ void mp9_march_delta_int(const int64_t* __restrict__ p, int ss,
-                                                    int64_t* __restrict__ out, int ostep) {
+template <int NC, typename Cells>
+__device__ __forceinline__ void mp9_march_delta(Cells p, int ss, int64_t* __restrict__ out, int ostep) {
   constexpr int NB = NC >= 8 ? NC / 8 : 1;   // blocks of NU interfaces
   constexpr int NU = NC >= 8 ? 8 : NC;
   static_assert(NB * NU == NC, "whole blocks");
@@ -289,10 +319,29 @@ __device__ __forceinline__ void mp9_march_delta_int(const int64_t* __restrict__ 
   for (int b = 0; b < NB; ++b) {
     FDLB_STEP(0) FDLB_STEP(1) FDLB_STEP(2) FDLB_STEP(3)
     FDLB_STEP(4) FDLB_STEP(5) FDLB_STEP(6) FDLB_STEP(7)
-    p += 8 * ss;
+    p.p += 8 * ss;
     out += 8 * ostep;
   }
 #undef FDLB_STEP
+}
+template <int NC>
+__device__ __forceinline__ void mp9_march_delta_int(const int64_t* p, int ss, int64_t* out, int ostep) {
+  mp9_march_delta<NC>(IntCells{p}, ss, out, ostep);
+}
+
+// The scale (largest biased exponent) of the values that march reads for NC
+// cells, and whether fixed point takes the line.
+template <int NC>
+__device__ __forceinline__ bool scale_of_line(const double* p, int ss, int& emax) {
+  int mx = 0, mn = 0x7fffffff;
+#pragma unroll
+  for (int k = -4; k <= NC + 4; ++k) {
+    const int m = mag_word(p[k * ss]);
+    mx = mx < m ? m : mx;
+    if (k >= 1 && k <= NC) mn = m < mn ? m : mn;
+  }
+  emax = mx >> 20;
+  return takes_fixed_point(mx, mn);
 }
 
 // The same flux differences in binary64 (their bits), for tiles the
@@ -331,11 +380,12 @@ __device__ __noinline__ void mp9_march_delta_fp64(const double* p, int ss, int64
   }
 }
 
-// |cx| dx + |cy| dy of flux differences given as binary64 bits.  A call, so
-// that the compiler does not run its binary64 operations beside the
-// fixed-point ones and select.
-__device__ __noinline__ double advection_bits(double cx, double cy, int64_t dx, int64_t dy) {
-  return fma(fabs(cy), dfrom(dy), fabs(cx) * dfrom(dx));
+// |cx| dx + |cy| dy of flux differences of which one or both are binary64 bits
+// (exponent 0).  A call, so that the compiler does not run its binary64
+// operations beside the fixed-point ones and select.
+__device__ __noinline__ double advection_fp64(double cx, double cy, int64_t dx, int ex, int64_t dy, int ey) {
+  const double x = ex ? q_to_double(dx, ex) : dfrom(dx), y = ey ? q_to_double(dy, ey) : dfrom(dy);
+  return fma(fabs(cy), y, fabs(cx) * x);
 }
 
 }  // namespace fdlb

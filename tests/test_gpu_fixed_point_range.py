@@ -7,9 +7,10 @@ the step is homogeneous of degree one), and n with the oracle on the cells the
 jump's windows don't reach.
 
 Tolerance.  Where the fixed-point march runs, a cell lies at most 16 times
-below its tile's largest, so a flux difference is within 62 units of 2^-59 of
-32 times the cell's value (the power of two above the largest): 3.5e-15.  The
-binary64 march's own error is below 64 rounding units of it, 0.7e-14.  Three
+below the largest value its line reads, so a flux difference is within 62 units
+of 2^-59 of 32 times the cell's value (the power of two above the largest):
+3.5e-15.  The binary64 march's own error is below 64 rounding units of it,
+0.7e-14.  Three
 stages with two axes, each times dt |p| / ds < 0.1 and relaxed (u and T lose
 up to another factor of 10 to the moments' cancellations): 1e-13 for n, 1e-12
 for u and T, in place of which the march on one scale for all cells loses

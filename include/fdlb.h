@@ -238,7 +238,8 @@ int fdlb_batch_offsets(const fdlb_ctx* ctx, int64_t* base);
  * be NULL).  Allocates one temporary state copy. */
 int fdlb_autotune(fdlb_ctx* ctx, int trial_steps, int* variant_out, int* ctas_per_sm_out);
 
-/* Set the batch tile shape directly (variant 0, 1, 2 = 127, 63, 255 cells). */
+/* Set the batch tile shape directly (variant 0, 1, 2 = 127, 63, 255 cells;
+ * 1 to 64 CTAs per SM, 16 as fdlb_autotune returns it: a CTA per tile). */
 int fdlb_batch_set_tiling(fdlb_ctx* ctx, int variant, int ctas_per_sm);
 
 /* ---- adjoint (1-D binary64 contexts with outlet ghosts and Table I) --------

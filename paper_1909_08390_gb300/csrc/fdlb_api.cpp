@@ -980,9 +980,10 @@ int fdlb_batch_offsets(const fdlb_ctx* c, int64_t* base) {
   return FDLB_OK;
 }
 
-// CTAs per SM that the autotuner's grid size k stands for: the largest is a
-// CTA per tile (64 per SM at most), as a context starts with.
-static int tuned_ctas(int k) { return k >= 16 ? 64 : k; }
+// CTAs per SM that a grid size k of the autotuner and of fdlb_batch_set_tiling
+// stands for: its largest, 16, is a CTA per tile (64 per SM at most), as a
+// context starts with.
+static int tuned_ctas(int k) { return k == 16 ? 64 : k; }
 
 int fdlb_autotune(fdlb_ctx* c, int trial_steps, int* variant_out, int* ctas_per_sm_out) {
   if (!c) return set_err(nullptr, FDLB_EINVAL, "ctx is NULL");
@@ -1057,7 +1058,7 @@ int fdlb_batch_set_tiling(fdlb_ctx* c, int variant, int ctas_per_sm) {
   if (variant < 0 || variant >= fdlb::kBatchVariants || ctas_per_sm < 1 || ctas_per_sm > 64)
     return set_err(c, FDLB_EINVAL, "variant in [0, %d), ctas_per_sm in [1, 64]", fdlb::kBatchVariants);
   c->dp.variant = variant;
-  c->dp.bgrid = ctas_per_sm * c->nsm;
+  c->dp.bgrid = tuned_ctas(ctas_per_sm) * c->nsm;
   drop_graph(c);
   return upload_work(c);
 }
